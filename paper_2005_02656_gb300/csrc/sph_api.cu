@@ -365,7 +365,7 @@ int sph_init(const sph_params* params, int64_t n_max, sph_ctx** out) {
   ALLOC(ctx->nn, n);
   ALLOC(ctx->nbr, (size_t)mb * n);
   if (params->precision == SPH_FP64) ALLOC(ctx->wcache, (size_t)mb * n);
-  ALLOC(ctx->vol, 5 * n);
+  ALLOC(ctx->vol, 6 * n);
   ALLOC(ctx->rec_d, n);
   ALLOC(ctx->rec_i, n);
   ALLOC(ctx->rec_m, 5 * n);
@@ -394,10 +394,7 @@ int sph_init(const sph_params* params, int64_t n_max, sph_ctx** out) {
     for (int k = 0; k < 13; ++k) *f[k] = sbuf + (size_t)k * n;
     ctx->s.id = ctx->s_id_buf;
   }
-  if (ctx->vol) {
-    ctx->X = ctx->vol + n;
-    ctx->inv_rho = ctx->vol + 2 * n;
-  }
+  if (ctx->vol) ctx->X = ctx->vol + n;
   if (rc == SPH_OK) {
     e = cudaMemset(ctx->err, 0, sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(ctx->red.counter, 0, 8 * sizeof(unsigned int));

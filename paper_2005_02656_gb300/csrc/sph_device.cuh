@@ -307,6 +307,38 @@ __device__ __forceinline__ float f32_rn(double d) {
   return __int_as_float(f | (hi & 0x80000000u));                             // the exponent
 }
 
+// --- FP64 reciprocal square root ---
+// 1 / sqrt(x) = y0 (1 + q) for x > 0: y0 from the FP32 unit (relative error
+// below 2^-21), q = e/2 + 3 e^2/8 with e = 1 - x y0^2.  The e^2 term needs FP32
+// only, and the conversions between the formats run on the integer pipes, so
+// this takes 3 FP64 operations (the product with 1 + q is the caller's) where
+// rsqrt takes 6.  Values near the ends of the exponent range take rsqrt.
+__device__ __forceinline__ void root_parts(double x, double& y0, double& q) {
+  const uint32_t h = (uint32_t)__double2hiint(x);
+  const int ex = (int)(h >> 20) - 1023;
+  if (ex < -1000 || ex > 1000) {
+    y0 = rsqrt(x);
+    q = 0.0;
+    return;
+  }
+  const int odd = ex & 1;
+  const float m = __uint_as_float(((uint32_t)(127 + odd) << 23) | ((h & 0xfffffu) << 3) |
+                                  ((uint32_t)__double2loint(x) >> 29));
+  const uint32_t yb = __float_as_uint(rsqrtf(m));
+  y0 = __hiloint2double((int)((yb >> 3) + ((uint32_t)(896 - ((ex - odd) >> 1)) << 20)),
+                        (int)(yb << 29));
+  const double e = fma(-(x * y0), y0, 1.0);
+  const uint32_t eh = (uint32_t)__double2hiint(e) & 0x7fffffffu;
+  const float ef = __uint_as_float((max(eh, 897u << 20) - (896u << 20)) << 3);
+  const uint32_t sb = __float_as_uint(0.375f * ef * ef);
+  q = fma(0.5, e, __hiloint2double((int)((sb >> 3) + (896u << 20)), (int)(sb << 29)));
+}
+__device__ __forceinline__ double inv_root(double x) {
+  double y0, q;
+  root_parts(x, y0, q);
+  return fma(y0, q, y0);
+}
+
 // --- reductions ---
 __device__ __forceinline__ double warp_min(double v) {
   for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));

@@ -107,16 +107,17 @@ struct sph_ctx {
   int32_t* nn;
   uint32_t* nbr;
 
-  // FP64 path: W_ab(h_a) of every list entry, written by the density pass and
+  // FP64 path: h_a^3 W_ab(h_a) / B_n of every list entry, written by the density pass and
   // read by IAD and momentum (nbr layout; allocated for SPH_FP64 contexts)
   double* wcache;
 
-  // FP64 per-particle helpers: one block of 5 * n_max doubles
+  // FP64 per-particle helpers: one block of 6 * n_max doubles
   double* vol;          // m / rho          (vol + 0 n_max)
   double* X;            // P / rho^2        (vol + 1 n_max)
-  double* inv_rho;      // 1 / rho          (vol + 2 n_max)
+                        // alpha / (4 rho)  (vol + 2 n_max)
                         // 1 / h^2          (vol + 3 n_max)
-                        // B_n / h^3        (vol + 4 n_max)
+                        // m B_n / h^3      (vol + 4 n_max)
+                        // B_n / h^3        (vol + 5 n_max)
 
   // FP32 mixed-path per-particle records (sorted order, sph_pairs_fp32.cu)
   float4* rec_d;        // offset x, y, z, m               (gather)

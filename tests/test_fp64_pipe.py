@@ -1,0 +1,110 @@
+"""The FP64 kernels' work outside the FP64 pipe: the fixed-point kernel series
+(sph_fixed.cuh, compiled for the CPU), and the FP64 pair sums at the particle
+counts where their lane split changes."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import sph_inputs
+from helpers import field_errors, oracle_outputs
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2005_02656_gb300", "csrc")
+
+WRAP = """
+#include "sph_fixed.cuh"
+extern "C" void eval(const double* t, double* s, double* s6, double* d, long n) {
+  for (long i = 0; i < n; ++i) {
+    s[i] = sph::fx::S(t[i]);
+    double w;
+    sph::fx::S6_d(t[i], w, d[i]);
+    s6[i] = sph::fx::S6(t[i]);
+    if (w != s6[i]) s6[i] = -1.0;
+  }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def fixed(tmp_path_factory):
+    d = tmp_path_factory.mktemp("fx")
+    src, lib = d / "fx.cpp", d / "fx.so"
+    src.write_text(WRAP)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-o", str(lib),
+                    str(src)], check=True)
+    f = C.CDLL(str(lib))
+
+    def run(t):
+        t = np.ascontiguousarray(t, dtype=np.float64)
+        out = [np.empty_like(t) for _ in range(3)]
+        f.eval(*[a.ctypes.data_as(C.c_void_p) for a in (t, *out)], C.c_long(t.size))
+        return out
+    return run
+
+
+def _series(t, k0):
+    """sum_{k >= k0} of the Maclaurin series of sin(x)/x (k0 = 0) or of its t-derivative
+    (k0 = 1) at x^2 = (pi/2)^2 t, by mpmath."""
+    mp = pytest.importorskip("mpmath")
+    mp.mp.dps = 40
+    S = [mp.sin(mp.pi / 2 * mp.sqrt(v)) / (mp.pi / 2 * mp.sqrt(v)) if v else mp.mpf(1)
+         for v in map(mp.mpf, t)]
+    if k0 == 0:
+        return S
+    return [(mp.cos(mp.pi / 2 * mp.sqrt(v)) - s) / (2 * v) if v > 1e-8 else -mp.pi ** 2 / 24
+            for v, s in zip(map(mp.mpf, t), S)]
+
+
+def test_fixed_point_series(fixed):
+    """|S error| <= 2^-60 (14 truncated products of at most 3 units of 2^-64 each, a factor of
+    at most 2 between the formats, y < 1) plus the rounding of the double; S^6 and its
+    derivative likewise, relative to S^5."""
+    rng = np.random.default_rng(1)
+    t = np.concatenate([rng.uniform(0, 4, 400), 4 - 2.0 ** -rng.uniform(0, 51, 200),
+                        2.0 ** -rng.uniform(0, 80, 200)])
+    s, s6, d = fixed(t)
+    S, dS = _series(t, 0), _series(t, 1)
+    for i in range(t.size):
+        e = 2.0 ** -60
+        assert abs(s[i] - S[i]) <= e + 2.0 ** -53 * S[i], t[i]
+        assert abs(s6[i] - S[i] ** 6) <= 6 * (S[i] + e) ** 5 * e + 2.0 ** -52 * S[i] ** 6, t[i]
+        ref = 6 * S[i] ** 5 * dS[i]
+        if t[i] > 1e-8:
+            assert abs(d[i] - ref) <= 40 * (S[i] + e) ** 4 * e + 2.0 ** -51 * abs(ref), t[i]
+
+
+def test_fixed_point_edges(fixed):
+    """The origin, tiny arguments, the support's edge and beyond, infinity and NaN."""
+    t = np.array([0.0, 5e-324, 1e-300, 4.0, 4.0 + 1e-15, 1e300, np.inf, np.nan])
+    s, s6, d = fixed(t)
+    np.testing.assert_array_equal(s, [1, 1, 1, 0, 0, 0, 0, 0])
+    np.testing.assert_array_equal(s6, [1, 1, 1, 0, 0, 0, 0, 0])
+    np.testing.assert_allclose(d[:3], -np.pi ** 2 / 4, rtol=1e-15)
+    np.testing.assert_array_equal(d[3:], 0)
+    s, s6, _ = fixed([np.nextafter(4.0, 0.0)])
+    assert 0 <= s6[0] <= 1e-90 and 0 <= s[0] < 1e-15
+
+
+# particles per target-lane split: 16 lanes (below 16,384), 8, 4 (from 131,072)
+@pytest.mark.gpu
+@pytest.mark.parametrize("side,gradh", [(7, 0), (25, 1), (26, 0), (50, 0), (51, 1)])
+def test_fp64_lane_splits(side, gradh):
+    """FP64 fields against the oracle at both sides of each split (the parity bound 1e-12)."""
+    from paper_2005_02656_gb300 import SphSim
+    s = sph_inputs.jittered_box(side, seed_index=40 + side)
+    rc, _, ref = oracle_outputs(s, ng_target=0, gradh=gradh)
+    assert rc == 0
+    sim = SphSim(s, gradh=gradh, ng_target=0)
+    sim.find_neighbors()
+    sim.density()
+    sim.iad()
+    sim.momentum_energy()
+    got = sim.to_numpy()
+    assert sim.error_word() == 0
+    sim.close()
+    e = field_errors(got, ref)
+    for k in ("rho", "p", "c", "iad", "a", "du"):
+        assert e[k] <= 1e-12, (k, e)
