@@ -182,120 +182,12 @@ __device__ __forceinline__ bool accept64(const Node& nd, const double p[3], doub
   return !inside && nd.size < theta * R;
 }
 
-// The walk of a warp: 32 consecutive sorted particles (one lane each) share
-// one depth-first stack whose entries carry the mask of lanes that reached
-// the node through nodes they opened.  Every lane still takes its own
-// decisions and sees its nodes in its own depth-first order (so the result
-// equals a walk per particle), but node and particle loads are common to the
-// warp and an opened leaf is summed by all its lanes in lockstep.
 constexpr int kWalkWarps = 4;
 
-__global__ void __launch_bounds__(32 * kWalkWarps) k_walk(const Node* nodes, int32_t root,
-                                                          StateView s, int64_t n, double G,
-                                                          double eps, double theta, double* gx,
-                                                          double* gy, double* gz,
-                                                          unsigned long long* stats,
-                                                          uint32_t* err) {
-  __shared__ int32_t st_node[kWalkWarps][kStack];
-  __shared__ uint32_t st_mask[kWalkWarps][kStack];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  unsigned long long nodes_used = 0, pairs = 0;
-  const double eps2 = eps * eps;
-  const int64_t tiles = (n + 31) / 32;
-  for (int64_t tile = blockIdx.x * (int64_t)kWalkWarps + w; tile < tiles;
-       tile += (int64_t)gridDim.x * kWalkWarps) {
-    const int64_t a = tile * 32 + lane;
-    const bool valid = a < n;
-    const double p[3] = {valid ? s.x[a] : 0.0, valid ? s.y[a] : 0.0, valid ? s.z[a] : 0.0};
-    double acc[3] = {0.0, 0.0, 0.0};
-    int sp = 0;
-    const uint32_t all = __ballot_sync(0xffffffffu, valid);
-    if (lane == 0) {
-      st_node[w][0] = root;
-      st_mask[w][0] = all;
-    }
-    sp = 1;
-    __syncwarp();
-    bool overflow = false;
-    while (sp > 0) {
-      --sp;
-      const int32_t k = st_node[w][sp];
-      const uint32_t mask = st_mask[w][sp];
-      __syncwarp();
-      const Node& nd = nodes[k];
-      const bool live = (mask >> lane) & 1u;
-      bool open = false;
-      if (live) {
-        double r[3], R2, R;
-        if (accept64(nd, p, theta, r, R2, R)) {
-          // one reciprocal and one reciprocal square root per node: the FP64
-          // pipe runs divisions and square roots as multi-instruction sequences
-          const double inv_s = rsqrt(R2 + eps2);
-          const double mono = G * nd.M * (inv_s * inv_s * inv_s);
-          const double inv_R = 1.0 / R;
-          const double inv_R2 = inv_R * inv_R;
-          const double g5 = G * (inv_R2 * inv_R2 * inv_R);
-          const double* Q = nd.Q;
-          const double Qr[3] = {Q[0] * r[0] + Q[1] * r[1] + Q[2] * r[2],
-                                Q[1] * r[0] + Q[3] * r[1] + Q[4] * r[2],
-                                Q[2] * r[0] + Q[4] * r[1] + Q[5] * r[2]};
-          const double rQr = r[0] * Qr[0] + r[1] * Qr[1] + r[2] * Qr[2];
-          const double g7 = 2.5 * g5 * rQr * inv_R2;
-          for (int i = 0; i < 3; ++i) acc[i] += -mono * r[i] + g5 * Qr[i] - g7 * r[i];
-          ++nodes_used;
-        } else {
-          open = true;
-        }
-      }
-      const uint32_t omask = __ballot_sync(0xffffffffu, open);
-      if (omask == 0) continue;
-      if (nd.first < 0) {
-        // an opened leaf: its particles, in order, for the lanes that opened it
-        for (int32_t b = nd.p0; b < nd.p0 + nd.np; ++b) {
-          const double xb = s.x[b], yb = s.y[b], zb = s.z[b], mb = s.m[b];
-          if (open && b != a) {
-            const double d[3] = {p[0] - xb, p[1] - yb, p[2] - zb};
-            const double inv = rsqrt((d[0] * d[0] + d[1] * d[1]) + d[2] * d[2] + eps2);
-            const double f = G * mb * (inv * inv * inv);
-            for (int q = 0; q < 3; ++q) acc[q] -= f * d[q];
-            ++pairs;
-          }
-        }
-      } else {
-        if (sp + nd.nchild > kStack) {  // cannot happen for <= 8 Morton bits; kept as a guard
-          overflow = true;
-          break;
-        }
-        if (lane == 0)
-          for (int j = nd.nchild - 1, q = sp; j >= 0; --j, ++q) {
-            st_node[w][q] = nd.first + j;
-            st_mask[w][q] = omask;
-          }
-        sp += nd.nchild;
-        __syncwarp();
-      }
-    }
-    if (overflow && lane == 0) raise_flag(err, SPH_FLAG_CELL_OVERFLOW);
-    if (valid) {
-      gx[a] = acc[0];
-      gy[a] = acc[1];
-      gz[a] = acc[2];
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    nodes_used += __shfl_xor_sync(0xffffffffu, nodes_used, o);
-    pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
-  }
-  if (lane == 0) {
-    atomicAdd(stats, nodes_used);
-    atomicAdd(stats + 1, pairs);
-  }
-}
-
-// ---- FP32-mixed walk ------------------------------------------------------
-// The node and particle terms in FP32, the opening decisions exact, and no
-// FP64 operation inside the walk (the FP64 pipe runs at 1/64 of the FP32
-// rate).  Coordinates are taken relative to the grid origin lo and split into
+// ---- opening decisions in FP32 --------------------------------------------
+// FP64 runs at 1/64 of the FP32 rate on this part, so both walks decide in
+// FP32, exactly (accept_mixed), and the FP32-mixed one evaluates its terms in
+// FP32 as well.  Coordinates are taken relative to the grid origin lo and split into
 // an FP32 head and tail (v = hi + lo to about 2^-48 |v|), so r = x_a - c is
 // (hi_a - hi_c) + (lo_a - lo_c) with FP32 rounding relative to |r| instead of
 // to the box.  Each particle is stored relative to its leaf's centre of mass,
@@ -315,22 +207,23 @@ __device__ __forceinline__ void split2(double v, float& hi, float& lo) {
   lo = (float)(v - (double)hi);
 }
 
-__global__ void k_nodes32(const Node* nodes, int64_t nn, double lx, double ly, double lz,
+// FP32 records of the nodes, coordinates and sizes scaled by `sc` (a power of two).
+__global__ void k_nodes32(const Node* nodes, int64_t nn, double lx, double ly, double lz, double sc,
                           NodeF* out) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nn;
        k += (int64_t)gridDim.x * blockDim.x) {
     const Node& nd = nodes[k];
     float ch[3], cl[3];
-    split2(nd.c[0] - lx, ch[0], cl[0]);
-    split2(nd.c[1] - ly, ch[1], cl[1]);
-    split2(nd.c[2] - lz, ch[2], cl[2]);
+    split2((nd.c[0] - lx) * sc, ch[0], cl[0]);
+    split2((nd.c[1] - ly) * sc, ch[1], cl[1]);
+    split2((nd.c[2] - lz) * sc, ch[2], cl[2]);
     NodeF f;
     f.cm = make_float4(ch[0], ch[1], ch[2], (float)nd.M);
-    f.q1 = make_float4((float)nd.Q[4], (float)nd.Q[5], (float)nd.size, cl[0]);
-    f.lo = make_float4((float)(nd.box_lo[0] - lx), (float)(nd.box_lo[1] - ly),
-                       (float)(nd.box_lo[2] - lz), cl[1]);
-    f.hi = make_float4((float)(nd.box_hi[0] - lx), (float)(nd.box_hi[1] - ly),
-                       (float)(nd.box_hi[2] - lz), cl[2]);
+    f.q1 = make_float4((float)nd.Q[4], (float)nd.Q[5], (float)(nd.size * sc), cl[0]);
+    f.lo = make_float4((float)((nd.box_lo[0] - lx) * sc), (float)((nd.box_lo[1] - ly) * sc),
+                       (float)((nd.box_lo[2] - lz) * sc), cl[1]);
+    f.hi = make_float4((float)((nd.box_hi[0] - lx) * sc), (float)((nd.box_hi[1] - ly) * sc),
+                       (float)((nd.box_hi[2] - lz) * sc), cl[2]);
     f.q0 = make_float4((float)nd.Q[0], (float)nd.Q[1], (float)nd.Q[2], (float)nd.Q[3]);
     f.t = make_int4(nd.first, nd.nchild, nd.p0, nd.np);
     out[k] = f;
@@ -351,19 +244,251 @@ __global__ void k_leaf_offsets(const Node* nodes, int64_t n_leaves, StateView s,
 // Constants of the FP32 walk, converted on the host.
 struct Walk32Consts {
   double lx, ly, lz;   // grid origin
+  double sc;           // scale of the FP32 coordinates, a power of two
   double theta;        // for the FP64 decision
   float G, eps2, th;
   float mb;            // box-face margin: covers the FP32 rounding of box and head
   float aL;            // absolute distance margin
 };
 
-// Same warp walk as k_walk.  The FP32 decision uses margins that cover the
+// Node k as a target at head ph and tail pl sees it.
+struct NodeSeen {
+  float4 cm, q1;
+  int4 t;
+  float r[3], R2, inv_R;
+};
+
+// The opening decision for one target, in FP32 with margins that cover the
 // rounding of the stored box faces and of the particle's head (each <= L
 // 2^-24, L the grid's largest extent) and of the FP32 distance (relative
-// 2^-22 with rsqrtf): mb on a box face, aL + 2e-6 R on the distance.  A lane
-// inside a margin takes the FP64 decision of k_walk (accept64 on the FP64
-// node), so every lane accepts and opens exactly the nodes that the FP64 walk
-// does.
+// 2^-22 with rsqrtf): mb on a box face, aL + 2e-6 R on the distance.  Inside a
+// margin, and wherever an FP32 value is not finite, the FP64 decision
+// (accept64 on the FP64 node) is taken, so the nodes accepted and opened are
+// exactly those of an FP64 walk.  `live`: false leaves the decision out.
+__device__ __forceinline__ bool accept_mixed(const Node* nodes, const NodeF* nf, int32_t k,
+                                             const float ph[3], const float pl[3], bool live,
+                                             const StateView& s, int64_t a,
+                                             const Walk32Consts& k32, NodeSeen& v) {
+  const NodeF* f = nf + k;
+  v.cm = __ldg(&f->cm);
+  v.q1 = __ldg(&f->q1);
+  const float4 blo = __ldg(&f->lo), bhi = __ldg(&f->hi);
+  v.t = __ldg(&f->t);
+  v.r[0] = (ph[0] - v.cm.x) + (pl[0] - v.q1.w);
+  v.r[1] = (ph[1] - v.cm.y) + (pl[1] - blo.w);
+  v.r[2] = (ph[2] - v.cm.z) + (pl[2] - bhi.w);
+  bool accept = false;
+  if (live) {
+    v.R2 = fmaf(v.r[2], v.r[2], fmaf(v.r[1], v.r[1], v.r[0] * v.r[0]));
+    v.inv_R = rsqrtf(v.R2);
+    const float Rf = v.R2 * v.inv_R;
+    const float size = v.q1.z, mb = k32.mb;
+    // the box: certainly outside, certainly inside, or within mb of a face.
+    // dmin is the smallest signed distance of the particle to a face
+    // (negative outside); its own rounding (<= L 2^-24) adds to the
+    // stored faces' and the head's, all within mb = 4 L 2^-24.
+    const float dmin =
+        fminf(fminf(fminf(ph[0] - blo.x, bhi.x - ph[0]), fminf(ph[1] - blo.y, bhi.y - ph[1])),
+              fminf(ph[2] - blo.z, bhi.z - ph[2]));
+    const bool out_c = dmin < -mb;
+    const bool in_c = dmin >= mb;
+    const bool acc_c = size * (1.f + 1e-6f) < k32.th * (Rf * (1.f - 2e-6f) - k32.aL);
+    const bool rej_c = size * (1.f - 1e-6f) > k32.th * (Rf * (1.f + 2e-6f) + k32.aL);
+    if (in_c || rej_c) {
+      accept = false;
+    } else if (out_c && acc_c) {
+      accept = true;
+    } else {
+      // FP64 positions are reloaded here rather than kept live across the walk
+      const double p[3] = {s.x[a], s.y[a], s.z[a]};
+      double r64[3], R2_64, R64;
+      accept = accept64(nodes[k], p, k32.theta, r64, R2_64, R64);
+    }
+  }
+  return accept;
+}
+
+// ---- FP64 walk ------------------------------------------------------------
+// A warp walks kTile64 consecutive targets together on one stack, with the
+// FP32 decisions of accept_mixed, and only queues what it accepts: per lane one
+// ring of accepted nodes and one of opened leaves in shared memory.  kLanes64
+// lanes share a target: they take the same decisions, and every kLanes64-th of
+// its node terms and leaf particles each, added at the end by a fixed butterfly.
+// The FP64 terms are evaluated from the rings, each lane taking its own next
+// term, so the FP64 pipe (which bounds the kernel, at 2 operations per clock
+// and SM; 86% busy) works on full warps: a warp that evaluates a term where it
+// meets it has 21 of its 32 lanes in it, because lanes that did not open the
+// parent or that open the node itself sit it out.  FP64 operations per node
+// term 42, per leaf particle 16 (G is applied once per target; inv_root).
+// Uniform sphere, theta = 0.5, whole call: 137,376 particles 28.6 -> 10.4 ms,
+// 2,176 particles 2.19 -> 0.63 ms (one lane per target and full rings: 12.5 and
+// 1.62 ms; 4 lanes: 10.4 and 0.78 ms).
+constexpr int kLanes64 = 8;
+constexpr int kTile64 = 32 / kLanes64;
+constexpr int kRing = 32;       // entries per lane and ring
+constexpr int kDrainLanes = 28; // evaluate while at least so many lanes hold a term
+
+__global__ void __launch_bounds__(32 * kWalkWarps) k_walk(const Node* nodes, const NodeF* nf,
+                                                          int32_t root, StateView s, int64_t n,
+                                                          Walk32Consts k32, double G, double eps2,
+                                                          double* gx, double* gy, double* gz,
+                                                          unsigned long long* stats,
+                                                          uint32_t* err) {
+  __shared__ int32_t st_node[kWalkWarps][kStack];
+  __shared__ uint32_t st_mask[kWalkWarps][kStack];
+  __shared__ int32_t ring_node[kWalkWarps][kRing][32];
+  __shared__ int32_t ring_leaf[kWalkWarps][kRing][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int sub = lane % kLanes64;
+  unsigned long long nodes_used = 0, pairs = 0;
+  const int64_t tiles = (n + kTile64 - 1) / kTile64;
+  for (int64_t tile = blockIdx.x * (int64_t)kWalkWarps + w; tile < tiles;
+       tile += (int64_t)gridDim.x * kWalkWarps) {
+    const int64_t a = tile * kTile64 + lane / kLanes64;
+    const bool valid = a < n;
+    const int32_t a32 = valid ? (int32_t)a : -1;
+    const double p[3] = {valid ? s.x[a] : 0.0, valid ? s.y[a] : 0.0, valid ? s.z[a] : 0.0};
+    float ph[3], pl[3];
+    split2((p[0] - k32.lx) * k32.sc, ph[0], pl[0]);
+    split2((p[1] - k32.ly) * k32.sc, ph[1], pl[1]);
+    split2((p[2] - k32.lz) * k32.sc, ph[2], pl[2]);
+    double acc[3] = {0.0, 0.0, 0.0};
+    uint32_t accepted = 0;
+    uint32_t n_in = 0, n_out = 0;      // ring positions: nodes queued and evaluated
+    uint32_t l_in = 0, l_out = 0;      // leaves queued and begun
+    int32_t cur = 0, end = 0;          // particles of the leaf under evaluation
+
+    // Evaluates queued node terms (a term of every lane that has one per turn):
+    // while at least `lanes` lanes take part, and `turns` turns in any case.
+    auto drain_nodes = [&](int lanes, int turns) {
+      for (;; --turns) {
+        const bool have = n_out != n_in;
+        const uint32_t m = __ballot_sync(0xffffffffu, have);
+        if (m == 0 || (turns <= 0 && __popc(m) < lanes)) break;
+        if (have) {
+          const Node& nd = nodes[ring_node[w][n_out % kRing][lane]];
+          ++n_out;
+          const double r[3] = {p[0] - nd.c[0], p[1] - nd.c[1], p[2] - nd.c[2]};
+          const double R2 = (r[0] * r[0] + r[1] * r[1]) + r[2] * r[2];
+          const double inv_R = inv_root(R2);
+          const double inv_s = eps2 > 0.0 ? inv_root(R2 + eps2) : inv_R;
+          const double mono = nd.M * (inv_s * inv_s * inv_s);
+          const double j2 = inv_R * inv_R;
+          const double g5 = j2 * j2 * inv_R;
+          const double* Q = nd.Q;
+          const double Qr[3] = {Q[0] * r[0] + Q[1] * r[1] + Q[2] * r[2],
+                                Q[1] * r[0] + Q[3] * r[1] + Q[4] * r[2],
+                                Q[2] * r[0] + Q[4] * r[1] + Q[5] * r[2]};
+          const double rQr = r[0] * Qr[0] + r[1] * Qr[1] + r[2] * Qr[2];
+          const double kr = fma(-2.5, g5 * (rQr * j2), -mono);
+          for (int i = 0; i < 3; ++i) acc[i] = fma(kr, r[i], fma(g5, Qr[i], acc[i]));
+        }
+      }
+    };
+    // The same for the particles of queued leaves, in order, the target left out.
+    auto drain_leaves = [&](int lanes, uint32_t room) {
+      for (;;) {
+        if (cur == a32) cur += kLanes64;
+        while (cur >= end && l_out != l_in) {
+          const int4 t = __ldg(&nf[ring_leaf[w][l_out % kRing][lane]].t);
+          ++l_out;
+          cur = t.z + sub == a32 ? a32 + kLanes64 : t.z + sub;
+          end = t.z + t.w;
+        }
+        const bool have = cur < end;
+        const uint32_t m = __ballot_sync(0xffffffffu, have);
+        const bool full = __any_sync(0xffffffffu, l_in - l_out > room);
+        if (m == 0 || (!full && __popc(m) < lanes)) break;
+        if (have) {
+          const int32_t b = cur;
+          cur += kLanes64;
+          const double d[3] = {p[0] - s.x[b], p[1] - s.y[b], p[2] - s.z[b]};
+          const double inv =
+              inv_root(fma(d[2], d[2], fma(d[1], d[1], fma(d[0], d[0], eps2))));
+          const double f = s.m[b] * (inv * inv * inv);
+          for (int q = 0; q < 3; ++q) acc[q] = fma(-f, d[q], acc[q]);
+          ++pairs;
+        }
+      }
+    };
+
+    int sp = 0;
+    const uint32_t all = __ballot_sync(0xffffffffu, valid);
+    if (lane == 0) {
+      st_node[w][0] = root;
+      st_mask[w][0] = all;
+    }
+    sp = 1;
+    __syncwarp();
+    bool overflow = false;
+    while (sp > 0) {
+      --sp;
+      const int32_t k = st_node[w][sp];
+      const uint32_t mask = st_mask[w][sp];
+      __syncwarp();
+      const bool live = (mask >> lane) & 1u;
+      NodeSeen v;
+      const bool accept = accept_mixed(nodes, nf, k, ph, pl, live, s, a, k32, v);
+      const bool open = live && !accept;
+      if (accept && (accepted++ % kLanes64 == (uint32_t)sub)) {
+        ring_node[w][n_in % kRing][lane] = k;
+        ++n_in;
+        ++nodes_used;
+      }
+      const uint32_t omask = __ballot_sync(0xffffffffu, open);
+      if (__any_sync(0xffffffffu, n_in - n_out == kRing)) drain_nodes(kDrainLanes, 1);
+      if (omask == 0) continue;
+      if (v.t.x < 0) {
+        if (open) {
+          ring_leaf[w][l_in % kRing][lane] = k;
+          ++l_in;
+        }
+        if (__any_sync(0xffffffffu, l_in - l_out == kRing)) drain_leaves(kDrainLanes, kRing - 1);
+      } else {
+        if (sp + v.t.y > kStack) {  // cannot happen for <= 8 Morton bits; kept as a guard
+          overflow = true;
+          break;
+        }
+        if (lane == 0)
+          for (int j = v.t.y - 1, q = sp; j >= 0; --j, ++q) {
+            st_node[w][q] = v.t.x + j;
+            st_mask[w][q] = omask;
+          }
+        sp += v.t.y;
+        __syncwarp();
+      }
+    }
+    drain_nodes(0, 0);
+    drain_leaves(0, kRing);
+    if (overflow && lane == 0) raise_flag(err, SPH_FLAG_CELL_OVERFLOW);
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+#pragma unroll
+      for (int o = kLanes64 / 2; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    if (valid && sub == 0) {
+      gx[a] = G * acc[0];
+      gy[a] = G * acc[1];
+      gz[a] = G * acc[2];
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    nodes_used += __shfl_xor_sync(0xffffffffu, nodes_used, o);
+    pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+  }
+  if (lane == 0) {
+    atomicAdd(stats, nodes_used);
+    atomicAdd(stats + 1, pairs);
+  }
+}
+
+// ---- FP32-mixed walk ------------------------------------------------------
+// The warp walk with the terms evaluated in FP32 where they are met: 32
+// consecutive sorted particles (one lane each) share one depth-first stack
+// whose entries carry the mask of lanes that reached the node through nodes
+// they opened.  Every lane takes its own decisions and sees its nodes in its
+// own depth-first order (so the result equals a walk per particle), but node
+// and particle loads are common to the warp and an opened leaf is summed by
+// all its lanes in lockstep.
 __global__ void __launch_bounds__(32 * kWalkWarps) k_walk32(const Node* nodes,
                                                             const NodeF* nf, const float4* po,
                                                             int32_t root, StateView s,
@@ -594,7 +719,7 @@ extern "C" int sph_gravity(sph_ctx* ctx, sph_state* state, double G, double eps,
   const size_t off_stats = off_part + sizeof(int64_t) * (size_t)nparts;
   const bool fp32 = ctx->prm.precision == SPH_FP32_MIXED;
   const size_t off_nf = (off_stats + 2 * sizeof(unsigned long long) + 127) & ~(size_t)127;
-  const size_t off_po = off_nf + (fp32 ? sizeof(sph::grav::NodeF) * (size_t)cap : 0);
+  const size_t off_po = off_nf + sizeof(sph::grav::NodeF) * (size_t)cap;
   const size_t bytes = off_po + (fp32 ? sizeof(float4) * (size_t)n : 0);
   int rc = grav_scratch(ctx, bytes);
   if (rc != SPH_OK) return rc;
@@ -636,33 +761,40 @@ extern "C" int sph_gravity(sph_ctx* ctx, sph_state* state, double G, double eps,
   const int64_t tiles = (n + 31) / 32;
   int wb = (int)((tiles + sph::grav::kWalkWarps - 1) / sph::grav::kWalkWarps);
   if (wb > sm * 256) wb = sm * 256;
+  sph::grav::NodeF* nf = (sph::grav::NodeF*)(base + off_nf);
+  double L = 0.0;
+  for (int ax = 0; ax < 3; ++ax) L = fmax(L, 1.001 * g.nc[ax] * g.cs[ax]);
+  // FP64 states may lie anywhere in the double range: their FP32 coordinates
+  // are scaled to [0, 2) by a power of two (exact); FP32-mixed ones are kept,
+  // as the terms use them
+  sph::grav::Walk32Consts k32;
+  k32.sc = fp32 || !(L > 0.0) || !isfinite(L) ? 1.0 : ldexp(1.0, -ilogb(L));
+  L *= k32.sc;
+  k32.lx = g.lo[0];
+  k32.ly = g.lo[1];
+  k32.lz = g.lo[2];
+  k32.theta = theta;
+  k32.G = (float)G;
+  k32.eps2 = (float)(eps * eps);
+  k32.th = (float)theta;
+  k32.mb = (float)(4.0 * L * 5.9604644775390625e-8);  // 4 L 2^-24
+  k32.aL = (float)(8.0 * L * 5.9604644775390625e-8);  // 8 L 2^-24
+  sph::grav::k_nodes32<<<sph::grav::blocks_for(noff, sm, 128), 128, 0, st>>>(
+      nodes, noff, g.lo[0], g.lo[1], g.lo[2], k32.sc, nf);
   if (fp32) {
-    sph::grav::NodeF* nf = (sph::grav::NodeF*)(base + off_nf);
     float4* po = (float4*)(base + off_po);
-    double L = 0.0;
-    for (int ax = 0; ax < 3; ++ax) L = fmax(L, 1.001 * g.nc[ax] * g.cs[ax]);
-    sph::grav::k_nodes32<<<sph::grav::blocks_for(noff, sm, 128), 128, 0, st>>>(
-        nodes, noff, g.lo[0], g.lo[1], g.lo[2], nf);
     sph::grav::k_leaf_offsets<<<sph::grav::blocks_for(n_occ, sm, 128), 128, 0, st>>>(
         nodes, n_occ, in, po);
-    sph::grav::Walk32Consts k32;
-    k32.lx = g.lo[0];
-    k32.ly = g.lo[1];
-    k32.lz = g.lo[2];
-    k32.theta = theta;
-    k32.G = (float)G;
-    k32.eps2 = (float)(eps * eps);
-    k32.th = (float)theta;
-    k32.mb = (float)(4.0 * L * 5.9604644775390625e-8);  // 4 L 2^-24
-    k32.aL = (float)(8.0 * L * 5.9604644775390625e-8);  // 8 L 2^-24
     sph::grav::k_walk32<<<wb, 32 * sph::grav::kWalkWarps, 0, st>>>(
         nodes, nf, po, root, in, n, k32, gx, gy, gz, stats, ctx->err);
     ctx->launches += 3;
   } else {
-    sph::grav::k_walk<<<wb, 32 * sph::grav::kWalkWarps, 0, st>>>(nodes, root, in, n, G, eps,
-                                                                 theta, gx, gy, gz, stats,
-                                                                 ctx->err);
-    ctx->launches += 1;
+    const int64_t tiles64 = (n + sph::grav::kTile64 - 1) / sph::grav::kTile64;
+    int wb64 = (int)((tiles64 + sph::grav::kWalkWarps - 1) / sph::grav::kWalkWarps);
+    if (wb64 > sm * 256) wb64 = sm * 256;
+    sph::grav::k_walk<<<wb64, 32 * sph::grav::kWalkWarps, 0, st>>>(
+        nodes, nf, root, in, n, k32, G, eps * eps, gx, gy, gz, stats, ctx->err);
+    ctx->launches += 2;
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return gfail(ctx, e, "sph_gravity launch");

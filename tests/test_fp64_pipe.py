@@ -1,6 +1,6 @@
 """The FP64 kernels' work outside the FP64 pipe: the fixed-point kernel series
-(sph_fixed.cuh, compiled for the CPU), and the FP64 pair sums at the particle
-counts where their lane split changes."""
+(sph_fixed.cuh, compiled for the CPU), and the FP64 pair sums and gravity walk at
+the particle counts where their lane split changes."""
 import ctypes as C
 import os
 import subprocess
@@ -8,6 +8,7 @@ import subprocess
 import numpy as np
 import pytest
 
+import oracle
 import sph_inputs
 from helpers import field_errors, oracle_outputs
 
@@ -108,3 +109,25 @@ def test_fp64_lane_splits(side, gradh):
     e = field_errors(got, ref)
     for k in ("rho", "p", "c", "iad", "a", "du"):
         assert e[k] <= 1e-12, (k, e)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("side,scale", [(5, 1.0), (9, 1e-25), (13, 1e25), (31, 1.0)])
+def test_fp64_gravity_scales(side, scale):
+    """The FP64 walk against the oracle's tree: ragged last tiles, and coordinates far outside
+    the FP32 range (its FP32 opening decisions work on scaled coordinates)."""
+    from paper_2005_02656_gb300 import Params, SphSim
+    s = sph_inputs.uniform_sphere(side, seed_index=90 + side)
+    for k in ("x", "y", "z", "h"):
+        s[k] = s[k] * scale
+    eps = 1e-3 * scale
+    sim = SphSim(s, Params(periodic=(0, 0, 0)))
+    g, counts = sim.gravity(1.0, eps, 0.5)
+    g, ids = g.cpu().numpy(), sim.t["id"].cpu().numpy()
+    assert sim.error_word() == 0
+    sim.close()
+    rc, ref, st = oracle.gravity_tree(s, eps=eps, theta=0.5)
+    assert rc == 0
+    ref = ref[np.argsort(s["id"])]
+    assert np.abs(g[np.argsort(ids)] - ref).max() <= 1e-12 * np.abs(ref).max()
+    np.testing.assert_array_equal(counts, st)
