@@ -20,11 +20,10 @@
 // particles 2.64, 3.77 and 14.5 ms, where the FP64 series, FP comparisons and
 // one thread per target took 7.38, 4.11 and 20.6 ms.
 #include <cuda_runtime.h>
-#include <type_traits>
-
 #include "sph_device.cuh"
 #include "sph_fixed.cuh"
 #include "sph_internal.cuh"
+#include "sph_lanes64.cuh"
 #include "sph_tile.cuh"
 
 namespace sph {
@@ -50,55 +49,10 @@ struct Lists64 {
   int max_nb;
 };
 
-// Periods of the minimum image: L per axis and the bit pattern of L / 2
-// (all ones on open axes, which no |d| exceeds).
-struct Image64 {
-  double L[3];
-  unsigned long long half[3];
-};
-
-__device__ __forceinline__ Image64 image_of(const Grid* g) {
-  Image64 im;
-#pragma unroll
-  for (int ax = 0; ax < 3; ++ax) {
-    im.L[ax] = g->Lbox[ax];
-    im.half[ax] = g->periodic[ax] ? (unsigned long long)__double_as_longlong(g->halfL[ax]) : ~0ull;
-  }
-  return im;
-}
-
-__device__ __forceinline__ bool beyond(double d, unsigned long long half) {
-  return ((unsigned long long)__double_as_longlong(d) & 0x7fffffffffffffffull) > half;
-}
-
-// FP64 minimum-image separation x_b - x_a: min_image's subtraction or addition
-// of the period where |d| > L/2, the test on the bit patterns of |d| and L/2
-// (ordered as the values are).  The FP64 additions sit behind a warp vote, so
-// that the warps away from the periodic boundaries skip them.
-__device__ __forceinline__ void sep64(const Image64& im, double& dx, double& dy, double& dz) {
-  const bool fx = beyond(dx, im.half[0]), fy = beyond(dy, im.half[1]), fz = beyond(dz, im.half[2]);
-  if (__any_sync(__activemask(), fx | fy | fz)) {
-    if (fx) dx += __double2hiint(dx) < 0 ? im.L[0] : -im.L[0];
-    if (fy) dy += __double2hiint(dy) < 0 ? im.L[1] : -im.L[1];
-    if (fz) dz += __double2hiint(dz) < 0 ? im.L[2] : -im.L[2];
-  }
-}
-
 // S(v)^n at t = v^2 by the context's kernel.
 __device__ __forceinline__ double shape64(double t, int n, const double2* tab) {
   if (tab) return kernel_w64_tab(t, 1.0, tab);
   return n == 6 ? fx::S6(t) : ipow(fx::S(t), n);
-}
-
-// Sum over the NSUB lanes of a target, left in sums[target of the block].
-// The per-target work around the pair loop (divisions, the matrix inverse: as
-// many FP64 instructions as a few pairs) then runs on whole warps, one thread
-// per target, instead of one lane in NSUB.
-template <int NSUB>
-__device__ __forceinline__ void lanes_sum(double v, double* sums) {
-#pragma unroll
-  for (int o = NSUB / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (threadIdx.x % NSUB == 0) sums[threadIdx.x / NSUB] = v;
 }
 
 // GRADH: also the grad-h terms, Omega_a = 1 + h_a/(3 rho_a) sum_b m_b dW/dh_a.
@@ -357,23 +311,6 @@ inline Lists64 lists64_of(sph_ctx* ctx) {
 
 inline unsigned blocks64(int64_t n, int nsub) {
   return (unsigned)((n * nsub + kThreads64 - 1) / kThreads64);
-}
-
-// Lanes per target.  More lanes keep the FP64 pipes of all SMs busy at small n
-// and cost lane sums and part-filled last turns of the lists at large n.
-// Density + IAD + momentum with 4 / 8 / 16 lanes (us): 1,728 particles 184 /
-// 109 / 88, 8,000: 250 / 241 / 234, 22,000: 610 / 569 / 575, 46,700: 1,084 /
-// 1,050 / 1,138, 1.07M: 21,560 / 22,070 / 24,120.
-inline int lanes64(int64_t n) { return n < 16384 ? 16 : n < 131072 ? 8 : 4; }
-
-// f(integral_constant<int, lanes>) for n particles.
-template <class F>
-inline void with_lanes64(int64_t n, F f) {
-  switch (lanes64(n)) {
-    case 4: f(std::integral_constant<int, 4>()); break;
-    case 8: f(std::integral_constant<int, 8>()); break;
-    default: f(std::integral_constant<int, 16>());
-  }
 }
 
 }  // namespace
