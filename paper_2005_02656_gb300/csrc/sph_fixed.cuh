@@ -140,5 +140,64 @@ SPH_FX void S6_d(double t, double& w, double& dw) {
   dw = -pack(d - (d >> 2), 7 - 5 * z);
 }
 
+// --- vectors in block fixed point ---
+// A vector's components share one power of two: component v is held as the
+// integer X = v 2^(N - e) (rounded toward zero), 2^e above every |v|, N = 61 (60
+// for the matrices), and used in two signed limbs, X = 2^32 h + l exactly.  A scalar product
+// of two such vectors is then nine 32-bit multiply-adds into two 64-bit sums,
+// with no carries: |X| < 2^61 leaves room for three terms.
+
+// Power of two above |v| for finite v, as the exponent field of a double plus
+// one (v = 0 and subnormal v give 1 and are taken as zero by fixed()).
+SPH_FX int exp_above(double v) { return (int)((bits_of(v) >> 52) & 0x7ffu) + 1; }
+
+// v 2^(N - (eb - 1023)), |v| < 2^(eb - 1023); subnormals give zero.
+template <int N>
+SPH_FX int64_t fixed(double v, int eb) {
+  const uint64_t b = bits_of(v);
+  const int s = eb - (int)((b >> 52) & 0x7ffu);  // >= 1
+  uint64_t m = (b & 0xfffffffffffffu) << (N - 52) | (uint64_t)1 << N;
+  m >>= (unsigned)s < 63u ? s : 63;  // |v| beyond the power of two: no value, but no overflow
+  const int64_t g = (int64_t)b >> 63;
+  return ((int64_t)m ^ g) - g;
+}
+
+struct Vec3 {
+  int32_t h[3];
+  int32_t l[3];
+};
+
+SPH_FX void put(Vec3& v, int i, int64_t x) {
+  v.l[i] = (int32_t)x;
+  v.h[i] = (int32_t)(x >> 32) - (v.l[i] >> 31);
+}
+
+// sum_i A_i B_i / 2^62 for |A_i|, |B_i| < 2^61, the products of the low limbs
+// left out (at most 3 units, of either sign) and the rest rounded.
+SPH_FX int64_t dot(const Vec3& a, const Vec3& b) {
+  int64_t hh = (int64_t)a.h[0] * b.h[0];
+  int64_t cr = (int64_t)a.h[0] * b.l[0];
+  cr += (int64_t)a.l[0] * b.h[0];
+  hh += (int64_t)a.h[1] * b.h[1];
+  cr += (int64_t)a.h[1] * b.l[1];
+  cr += (int64_t)a.l[1] * b.h[1];
+  hh += (int64_t)a.h[2] * b.h[2];
+  cr += (int64_t)a.h[2] * b.l[2];
+  cr += (int64_t)a.l[2] * b.h[2];
+  return (hh << 2) + ((cr + (1 << 29)) >> 30);
+}
+
+// The double nearest to x 2^k; zero where that is below the normal range.
+SPH_FX double scaled(int64_t x, int k) {
+  const int64_t g = x >> 63;
+  const uint64_t u = (uint64_t)((x ^ g) - g);
+  const int z = clz64(u);
+  const int f = 1085 + k - z;  // exponent field, less the implicit bit
+  if (u == 0 || f < 0) return 0.0;
+  const uint64_t m = u << z;
+  return from_bits((((uint64_t)(uint32_t)f << 52) + (m >> 11) + ((m >> 10) & 1u)) |
+                   ((uint64_t)g << 63));
+}
+
 }  // namespace fx
 }  // namespace sph

@@ -16,8 +16,8 @@
 //  - 1/r takes its seed from the FP32 reciprocal square root, and per-pair
 //    divisions are hoisted into per-particle arrays;
 //  - the per-target work runs on whole warps (lanes_sum).
-// Per pair 8 (density), 13 (IAD) and 64 (momentum) FP64 operations; at 1.07M
-// particles 2.64, 3.77 and 14.5 ms, where the FP64 series, FP comparisons and
+// Per pair 8 (density), 13 (IAD) and 37 (momentum) FP64 operations; at 1.07M
+// particles 2.64, 3.77 and 9.7 ms, where the FP64 series, FP comparisons and
 // one thread per target took 7.38, 4.11 and 20.6 ms.
 #include <cuda_runtime.h>
 #include "sph_device.cuh"
@@ -202,15 +202,77 @@ __global__ void __launch_bounds__(kThreads64) k_iad64(const Grid* gp, StateView 
   }
 }
 
+// Momentum's view of a neighbour, written per launch by k_pack64: 144 bytes read
+// as nine 16-byte loads where the separate arrays took 18 loads.
+struct alignas(16) Rec64 {
+  double x, y, z, hinv2;
+  double vx, vy, vz, c;
+  double m, mn;      // m, and m B_n / h^3 with the power of two of cf
+  double X, irq;
+  long long cf[6];   // C in block fixed point (fx::fixed), xx xy xz yy yz zz
+};
+
+// C (6 entries) as block fixed point; the exponent field of the power of two
+// above its largest entry, or 0 where an entry is not finite.
+__device__ __forceinline__ int fix_matrix(const double* C, long long cf[6]) {
+  int eb = 1;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) eb = max(eb, fx::exp_above(C[q]));
+#pragma unroll
+  for (int q = 0; q < 6; ++q) cf[q] = fx::fixed<60>(C[q], eb);
+  return eb <= 2047 ? eb : 0;
+}
+
+// 2^(eb - 1023) for eb of fix_matrix (not finite: NaN).
+__device__ __forceinline__ double power_of(int eb) {
+  if (eb == 0) return __longlong_as_double(0x7ff8000000000000LL);
+  return eb < 2047 ? __hiloint2double(eb << 20, 0) : 2.0 * __hiloint2double(2046 << 20, 0);
+}
+
+__global__ void k_pack64(StateView s, OutView o, Aux64 aux, int64_t n, Rec64* rec) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  Rec64 r;
+  r.x = s.x[i];
+  r.y = s.y[i];
+  r.z = s.z[i];
+  r.hinv2 = aux.hinv2[i];
+  r.vx = s.vx[i];
+  r.vy = s.vy[i];
+  r.vz = s.vz[i];
+  r.c = o.c[i];
+  r.m = s.m[i];
+  r.X = aux.X[i];
+  r.irq = aux.irq[i];
+  double C[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) C[q] = o.iad[6 * i + q];
+  r.mn = aux.mn[i] * power_of(fix_matrix(C, r.cf));
+  rec[i] = r;
+}
+
+// Rows of a symmetric matrix in block fixed point.
+__device__ __forceinline__ void rows(const long long cf[6], fx::Vec3 R[3]) {
+  constexpr int at[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) fx::put(R[i], j, cf[at[i][j]]);
+}
+
 // Per pair, with p_a = Pi / (2 rho_a) and p_b = Pi / (2 rho_b):
 //   a_a  -= m_b (W_a (X_a + p_a) C_a d + W_b (X_b + p_b) C_b d)
 //   du_a += m_b (W_a (X_a + p_a / 2) v_ab.C_a d + W_b p_b / 2 v_ab.C_b d)
 // The factor B_n/h_a^3 of W_a is applied to the sums, that of W_b carried by
-// m_b B_n/h_b^3.
+// m_b B_n/h_b^3.  C_a d, C_b d, v.C_a d, v.C_b d and x.v (27 of the 63 FP64
+// operations of a pair) are scalar products in block fixed point on the integer
+// pipes, d to the power of two above 2 h_a, v to its own: their rms error, about
+// 2^-60 of the largest components' product, is below FP64's.
 template <int NSUB>
-__global__ void __launch_bounds__(kThreads64) k_momentum64(const Grid* gp, StateView s, OutView o,
-                                                           Aux64 aux, Lists64 L, int64_t n,
-                                                           int sinc_n, uint32_t* err) {
+__global__ void __launch_bounds__(kThreads64) k_momentum64(const Grid* gp, const Rec64* rec,
+                                                           StateView s, OutView o, Aux64 aux,
+                                                           Lists64 L, int64_t n, int sinc_n,
+                                                           uint32_t* err) {
   constexpr int kT = kThreads64 / NSUB;  // targets of a block
   __shared__ double sums[4][kT];
   const Image64 im = image_of(gp);
@@ -218,61 +280,85 @@ __global__ void __launch_bounds__(kThreads64) k_momentum64(const Grid* gp, State
   const int64_t a_pair = blockIdx.x * (int64_t)kT + threadIdx.x / NSUB;
   const bool valid = a_pair < n;
   int64_t a = valid ? a_pair : n - 1;
-  const double xa = s.x[a], ya = s.y[a], za = s.z[a];
-  const double vxa = s.vx[a], vya = s.vy[a], vza = s.vz[a];
-  const double Xa = aux.X[a], ira = aux.irq[a], ca = o.c[a];
-  const double* Ca = o.iad + 6 * a;
-  const double a00 = Ca[0], a01 = Ca[1], a02 = Ca[2], a11 = Ca[3], a12 = Ca[4], a22 = Ca[5];
+  const Rec64* ra = rec + a;
+  const double xa = ra->x, ya = ra->y, za = ra->z;
+  const double vxa = ra->vx, vya = ra->vy, vza = ra->vz;
+  const double Xa = ra->X, ira = ra->irq, ca = ra->c;
+  const int ed = fx::exp_above(2.0 * s.h[a]);  // |d| < 2 h_a
+  fx::Vec3 Ca[3];
+  rows(ra->cf, Ca);
   const int cnt = valid ? min(L.nn[a], L.max_nb) : 0;
   const uint32_t* list = L.nbr + a * L.max_nb;
   const double* wrow = L.w + a * L.max_nb;
   double accx = 0, accy = 0, accz = 0, du = 0;      // terms of W_a, without B_n/h_a^3
   double bccx = 0, bccy = 0, bccz = 0, dub = 0;     // terms of W_b
   for (int k = sub; k < cnt; k += NSUB) {
-    const int64_t b = entry_index(list[k]);
-    double dx = s.x[b] - xa, dy = s.y[b] - ya, dz = s.z[b] - za;
+    const Rec64* rb = rec + entry_index(list[k]);
+    double dx = rb->x - xa, dy = rb->y - ya, dz = rb->z - za;
     sep64(im, dx, dy, dz);
     const double r2 = dx * dx + dy * dy + dz * dz;
-    const double vabx = vxa - s.vx[b], vaby = vya - s.vy[b], vabz = vza - s.vz[b];
-    const double xv = -(dx * vabx + dy * vaby + dz * vabz);  // x_ab . v_ab
+    const double vx = vxa - rb->vx, vy = vya - rb->vy, vz = vza - rb->vz;
+    fx::Vec3 D, V;
+    fx::put(D, 0, fx::fixed<61>(dx, ed));
+    fx::put(D, 1, fx::fixed<61>(dy, ed));
+    fx::put(D, 2, fx::fixed<61>(dz, ed));
+    const int ev = max(fx::exp_above(vx), max(fx::exp_above(vy), fx::exp_above(vz)));
+    fx::put(V, 0, fx::fixed<61>(vx, ev));
+    fx::put(V, 1, fx::fixed<61>(vy, ev));
+    fx::put(V, 2, fx::fixed<61>(vz, ev));
+    const double vnan = ev <= 2047 ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
+    const int64_t vd = fx::dot(V, D);  // -x_ab . v_ab
     double pa = 0.0, pb = 0.0;
-    if (okey(xv, 0) < 0) {  // xv < 0, decided on the integer pipes
+    if (vd > 0) {
+      const double xv = fx::scaled(-vd, ev + ed - 2 * 1023 - 60);
       double y0, e;
       root_parts(r2, y0, e);
       const double z = xv * y0, w = fma(z, e, z);
-      const double q = w * fma(3.0, w, -(ca + o.c[b]));
+      const double q = w * fma(3.0, w, -(ca + rb->c));
       pa = q * ira;
-      pb = q * aux.irq[b];
+      pb = q * rb->irq;
     }
-    const double wa = s.m[b] * wrow[k];
-    const double wb = aux.mn[b] * shape64(r2 * aux.hinv2[b], sinc_n, aux.ktab);
-    // C_a d (with B_n/h_a^3) and C_b d, d = x_b - x_a
-    const double Cadx = a00 * dx + a01 * dy + a02 * dz;
-    const double Cady = a01 * dx + a11 * dy + a12 * dz;
-    const double Cadz = a02 * dx + a12 * dy + a22 * dz;
-    const double* Cb = o.iad + 6 * b;
-    const double b00 = Cb[0], b01 = Cb[1], b02 = Cb[2], b11 = Cb[3], b12 = Cb[4], b22 = Cb[5];
-    const double Cbdx = b00 * dx + b01 * dy + b02 * dz;
-    const double Cbdy = b01 * dx + b11 * dy + b12 * dz;
-    const double Cbdz = b02 * dx + b12 * dy + b22 * dz;
+    const double wa = rb->m * wrow[k];
+    const double wb = rb->mn * shape64(r2 * rb->hinv2, sinc_n, aux.ktab);
     const double fa = wa * (Xa + pa);
-    const double fb = wb * (aux.X[b] + pb);
-    accx += fa * Cadx;
-    accy += fa * Cady;
-    accz += fa * Cadz;
-    bccx += fb * Cbdx;
-    bccy += fb * Cbdy;
-    bccz += fb * Cbdz;
-    const double vCa = vabx * Cadx + vaby * Cady + vabz * Cadz;
-    const double vCb = vabx * Cbdx + vaby * Cbdy + vabz * Cbdz;
-    du += wa * fma(0.5, pa, Xa) * vCa;
-    dub += wb * pb * vCb;
+    const double fb = wb * (rb->X + pb);
+    {
+      int64_t U[3];
+      fx::Vec3 Uv;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        U[i] = fx::dot(Ca[i], D);
+        fx::put(Uv, i, U[i]);
+      }
+      accx += fa * fx::scaled(U[0], 0);
+      accy += fa * fx::scaled(U[1], 0);
+      accz += fa * fx::scaled(U[2], 0);
+      du += wa * fma(0.5, pa, Xa) * (fx::scaled(fx::dot(V, Uv), ev - 1023) + vnan);
+    }
+    {
+      fx::Vec3 Cb[3], Uv;
+      rows(rb->cf, Cb);
+      int64_t U[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        U[i] = fx::dot(Cb[i], D);
+        fx::put(Uv, i, U[i]);
+      }
+      bccx += fb * fx::scaled(U[0], 0);
+      bccy += fb * fx::scaled(U[1], 0);
+      bccz += fb * fx::scaled(U[2], 0);
+      dub += wb * pb * fx::scaled(fx::dot(V, Uv), ev - 1023);
+    }
   }
-  const double norm = aux.wnorm[a];
-  lanes_sum<NSUB>(fma(-norm, accx, -bccx), sums[0]);
-  lanes_sum<NSUB>(fma(-norm, accy, -bccy), sums[1]);
-  lanes_sum<NSUB>(fma(-norm, accz, -bccz), sums[2]);
-  lanes_sum<NSUB>(fma(norm, du, 0.5 * dub), sums[3]);
+  // the powers of two of d, C_a and the products: C d = U 2^(e_C + e_d - 59),
+  // v.C d = R 2^(e_v + e_C + e_d - 58)
+  long long cf[6];
+  const double pd = power_of(ed) * 0x1p-59;
+  const double pn = aux.wnorm[a] * power_of(fix_matrix(o.iad + 6 * a, cf)) * pd;
+  lanes_sum<NSUB>(fma(-pn, accx, -pd * bccx), sums[0]);
+  lanes_sum<NSUB>(fma(-pn, accy, -pd * bccy), sums[1]);
+  lanes_sum<NSUB>(fma(-pn, accz, -pd * bccz), sums[2]);
+  lanes_sum<NSUB>(2.0 * fma(pn, du, 0.5 * pd * dub), sums[3]);
   __syncthreads();
   a = blockIdx.x * (int64_t)kT + threadIdx.x;
   if (threadIdx.x >= kT || a >= n) return;
@@ -339,12 +425,17 @@ void launch_iad_f64(sph_ctx* ctx, const StateView& s, const OutView& o, int64_t 
 
 void launch_momentum_f64(sph_ctx* ctx, const StateView& s, const OutView& o, int64_t n,
                          cudaStream_t st) {
+  // the records live in the hit-mask buffer of the FP32-mixed staged search
+  // (a search of either form writes its own before it is read)
+  static_assert(sizeof(Rec64) <= kMaskWords * sizeof(unsigned long long), "fits the mask buffer");
+  Rec64* rec = reinterpret_cast<Rec64*>(ctx->masks);
+  k_pack64<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(s, o, aux_of(ctx), n, rec);
   with_lanes64(n, [&](auto lanes) {
     constexpr int NS = decltype(lanes)::value;
     k_momentum64<NS><<<blocks64(n, NS), kThreads64, 0, st>>>(
-        ctx->grid, s, o, aux_of(ctx), lists64_of(ctx), n, (int)ctx->prm.sinc_n, ctx->err);
+        ctx->grid, rec, s, o, aux_of(ctx), lists64_of(ctx), n, (int)ctx->prm.sinc_n, ctx->err);
   });
-  ctx->launches += 1;
+  ctx->launches += 2;
 }
 
 }  // namespace sph

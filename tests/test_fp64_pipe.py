@@ -26,6 +26,22 @@ extern "C" void eval(const double* t, double* s, double* s6, double* d, long n) 
     if (w != s6[i]) s6[i] = -1.0;
   }
 }
+extern "C" void dots(const double* a, const double* b, double* out, long n) {
+  using namespace sph::fx;
+  for (long i = 0; i < n; ++i, a += 3, b += 3) {
+    int ea = 1, eb = 1;
+    for (int k = 0; k < 3; ++k) {
+      if (exp_above(a[k]) > ea) ea = exp_above(a[k]);
+      if (exp_above(b[k]) > eb) eb = exp_above(b[k]);
+    }
+    Vec3 A, B;
+    for (int k = 0; k < 3; ++k) {
+      put(A, k, fixed<60>(a[k], ea));
+      put(B, k, fixed<61>(b[k], eb));
+    }
+    out[i] = scaled(dot(A, B), ea + eb - 2 * 1023 - 59);
+  }
+}
 """
 
 
@@ -38,7 +54,11 @@ def fixed(tmp_path_factory):
                     str(src)], check=True)
     f = C.CDLL(str(lib))
 
-    def run(t):
+    def run(t, b=None):
+        if b is not None:
+            out = np.empty(len(t))
+            f.dots(*[v.ctypes.data_as(C.c_void_p) for v in (t, b, out)], C.c_long(len(t)))
+            return out
         t = np.ascontiguousarray(t, dtype=np.float64)
         out = [np.empty_like(t) for _ in range(3)]
         f.eval(*[a.ctypes.data_as(C.c_void_p) for a in (t, *out)], C.c_long(t.size))
@@ -87,6 +107,28 @@ def test_fixed_point_edges(fixed):
     np.testing.assert_array_equal(d[3:], 0)
     s, s6, _ = fixed([np.nextafter(4.0, 0.0)])
     assert 0 <= s6[0] <= 1e-90 and 0 <= s[0] < 1e-15
+
+
+def test_block_fixed_point_dot(fixed):
+    """Scalar products of vectors over many scales, with zero, tiny, subnormal and opposite
+    components.  Bound, in units of 2^-59 of the powers of two above the largest components:
+    3 (low limbs) + 1/2 (rounding) + 6 (two factors truncated by < 1 of 2^60 and 2^61 each, three
+    terms), and the rounding of the double."""
+    from fractions import Fraction
+    rng = np.random.default_rng(2)
+    n = 4000
+    a, b = (rng.normal(size=(n, 3)) * 2.0 ** rng.uniform(-200, 200, (n, 1)) for _ in range(2))
+    a[::7, 1] = 0.0
+    a[::11, 2] *= 1e-14
+    b[::13, 0] = 5e-324
+    b[::17] = np.cross(a[::17], b[::17])
+    b[::19] = 0.0
+    got = fixed(np.ascontiguousarray(a), np.ascontiguousarray(b))
+    for x, y, v in zip(a, b, got):
+        exact = sum(Fraction(p) * Fraction(q) for p, q in zip(x, y))
+        top = [2.0 ** (np.frexp(np.abs(w).max())[1]) for w in (x, y)]
+        bound = 9.5 * Fraction(top[0]) * Fraction(top[1]) / 2 ** 59
+        assert abs(Fraction(v) - exact) <= bound + abs(exact) / 2 ** 53, (x, y, v)
 
 
 # particles per target-lane split: 16 lanes (below 16,384), 8, 4 (from 131,072)
