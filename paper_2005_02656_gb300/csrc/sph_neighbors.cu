@@ -8,6 +8,7 @@
 
 #include "sph_device.cuh"
 #include "sph_internal.cuh"
+#include "sph_launch.cuh"
 #include "sph_find.cuh"
 #include "sph_tile.cuh"
 
@@ -27,6 +28,7 @@ __global__ void __launch_bounds__(kFindThreads, 1) k_find_tile(
     const Grid* gp, StateView s, const float4* __restrict__ pos32, const uint32_t* occ,
     const uint32_t* tbl_start, const uint32_t* tbl_count, int32_t* nn, uint32_t* nbr,
     int max_nb, uint32_t* err, unsigned long long* stats) {
+  dep_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   FindWarpSmem& W = reinterpret_cast<FindWarpSmem*>(smem_raw)[warp];
@@ -84,12 +86,12 @@ void launch_find_neighbors(sph_ctx* ctx, const StateView& s, int64_t n, cudaStre
                                                   smem);
     ctx->find_blocks = (per_sm > 0 ? per_sm : 1) * ctx->sm_count;
   }
-  k_find_tile<false><<<ctx->find_blocks, kFindThreads, smem, st>>>(
-      ctx->grid, s, ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr,
-      ctx->prm.max_nb, ctx->err, ctx->stats);
-  k_find_tile<true><<<ctx->find_blocks, kFindThreads, smem, st>>>(
-      ctx->grid, s, ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr,
-      ctx->prm.max_nb, ctx->err, ctx->stats);
+  launch_dep(k_find_tile<false>, ctx->find_blocks, kFindThreads, smem, st, ctx->grid, s,
+      ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb,
+      ctx->err, ctx->stats);
+  launch_dep(k_find_tile<true>, ctx->find_blocks, kFindThreads, smem, st, ctx->grid, s, ctx->pos32,
+      ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb, ctx->err,
+      ctx->stats);
   ctx->launches += 2;
 }
 

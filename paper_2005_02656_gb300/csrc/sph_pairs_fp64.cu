@@ -23,6 +23,7 @@
 #include "sph_device.cuh"
 #include "sph_fixed.cuh"
 #include "sph_internal.cuh"
+#include "sph_launch.cuh"
 #include "sph_lanes64.cuh"
 #include "sph_tile.cuh"
 
@@ -65,6 +66,7 @@ __global__ void __launch_bounds__(kThreads64) k_density64(const Grid* gp, StateV
                                                           Aux64 aux, Lists64 L, int64_t n,
                                                           double Bn, int sinc_n, double gamma,
                                                           double alpha, uint32_t* err) {
+  dep_enter();
   constexpr int kT = kThreads64 / NSUB;  // targets of a block
   __shared__ double sh_acc[kT], sh_g[GRADH ? kT : 1], sh_hinv2[kT];
   const Image64 im = image_of(gp);
@@ -136,6 +138,7 @@ __global__ void __launch_bounds__(kThreads64) k_density64(const Grid* gp, StateV
 template <int NSUB>
 __global__ void __launch_bounds__(kThreads64) k_iad64(const Grid* gp, StateView s, OutView o,
                                                       Aux64 aux, Lists64 L, int64_t n, uint32_t* err) {
+  dep_enter();
   constexpr int kT = kThreads64 / NSUB;  // targets of a block
   __shared__ double sums[6][kT];
   const Image64 im = image_of(gp);
@@ -230,6 +233,7 @@ __device__ __forceinline__ double power_of(int eb) {
 }
 
 __global__ void k_pack64(StateView s, OutView o, Aux64 aux, int64_t n, Rec64* rec) {
+  dep_enter();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   Rec64 r;
@@ -273,6 +277,7 @@ __global__ void __launch_bounds__(kThreads64) k_momentum64(const Grid* gp, const
                                                            StateView s, OutView o, Aux64 aux,
                                                            Lists64 L, int64_t n, int sinc_n,
                                                            uint32_t* err) {
+  dep_enter();
   constexpr int kT = kThreads64 / NSUB;  // targets of a block
   __shared__ double sums[4][kT];
   const Image64 im = image_of(gp);
@@ -406,9 +411,9 @@ void launch_density_f64(sph_ctx* ctx, const StateView& s, const OutView& o, int6
   with_lanes64(n, [&](auto lanes) {
     constexpr int NS = decltype(lanes)::value;
     auto kern = ctx->prm.gradh ? k_density64<NS, true> : k_density64<NS, false>;
-    kern<<<blocks64(n, NS), kThreads64, 0, st>>>(
-        ctx->grid, s, o, aux_of(ctx), lists64_of(ctx), n, ctx->Bn, (int)ctx->prm.sinc_n,
-        ctx->prm.gamma, ctx->prm.alpha, ctx->err);
+    launch_dep(kern, blocks64(n, NS), kThreads64, 0, st, ctx->grid, s, o, aux_of(ctx),
+        lists64_of(ctx), n, ctx->Bn, (int)ctx->prm.sinc_n, ctx->prm.gamma, ctx->prm.alpha,
+        ctx->err);
   });
   ctx->launches += 1;
 }
@@ -417,8 +422,8 @@ void launch_iad_f64(sph_ctx* ctx, const StateView& s, const OutView& o, int64_t 
                     cudaStream_t st) {
   with_lanes64(n, [&](auto lanes) {
     constexpr int NS = decltype(lanes)::value;
-    k_iad64<NS><<<blocks64(n, NS), kThreads64, 0, st>>>(ctx->grid, s, o, aux_of(ctx),
-                                                        lists64_of(ctx), n, ctx->err);
+    launch_dep(k_iad64<NS>, blocks64(n, NS), kThreads64, 0, st, ctx->grid, s, o, aux_of(ctx),
+        lists64_of(ctx), n, ctx->err);
   });
   ctx->launches += 1;
 }
@@ -429,11 +434,11 @@ void launch_momentum_f64(sph_ctx* ctx, const StateView& s, const OutView& o, int
   // (a search of either form writes its own before it is read)
   static_assert(sizeof(Rec64) <= kMaskWords * sizeof(unsigned long long), "fits the mask buffer");
   Rec64* rec = reinterpret_cast<Rec64*>(ctx->masks);
-  k_pack64<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(s, o, aux_of(ctx), n, rec);
+  launch_dep(k_pack64, (unsigned)((n + 127) / 128), 128, 0, st, s, o, aux_of(ctx), n, rec);
   with_lanes64(n, [&](auto lanes) {
     constexpr int NS = decltype(lanes)::value;
-    k_momentum64<NS><<<blocks64(n, NS), kThreads64, 0, st>>>(
-        ctx->grid, rec, s, o, aux_of(ctx), lists64_of(ctx), n, (int)ctx->prm.sinc_n, ctx->err);
+    launch_dep(k_momentum64<NS>, blocks64(n, NS), kThreads64, 0, st, ctx->grid, rec, s, o,
+        aux_of(ctx), lists64_of(ctx), n, (int)ctx->prm.sinc_n, ctx->err);
   });
   ctx->launches += 2;
 }

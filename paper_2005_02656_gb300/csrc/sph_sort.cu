@@ -21,6 +21,7 @@
 
 #include "sph_device.cuh"
 #include "sph_internal.cuh"
+#include "sph_launch.cuh"
 
 namespace sph {
 
@@ -44,6 +45,7 @@ __device__ __forceinline__ long long warp_max_ll(long long v) {
 // the open axes only (periodic axes take the box and keep the neutral keys).
 __global__ void k_grid_reduce(StateView in, int64_t n, sph_params prm, Grid* g, long long* part,
                               unsigned int* counter, uint32_t* err) {
+  dep_enter();
   __shared__ long long sh[kRedThreads / 32][7];
   __shared__ bool last;
   const bool open[3] = {!prm.periodic[0], !prm.periodic[1], !prm.periodic[2]};
@@ -151,6 +153,7 @@ __global__ void k_grid_reduce(StateView in, int64_t n, sph_params prm, Grid* g, 
 }
 
 __global__ void k_zero_table(const Grid* g, uint32_t* count, double* org) {
+  dep_enter();
   uint32_t size = g->tbl_size;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < size; i += gridDim.x * blockDim.x)
     count[i] = 0u;
@@ -181,6 +184,7 @@ __device__ __forceinline__ void cell_coords(const Grid& g, double x, double y, d
 
 __global__ void k_cell_count(StateView in, int64_t n, const Grid* gp, uint32_t* count,
                              uint32_t* code, uint32_t* slot) {
+  dep_enter();
   const Grid g = *gp;
   const int lane = threadIdx.x & 31;
   // the loop is warp-uniform (i - lane is the warp's first index); lanes past
@@ -213,6 +217,7 @@ constexpr int kScanThreads = 1024;
 constexpr int kPerThread = kScanItems / kScanThreads;
 
 __global__ void k_scan_a(const Grid* g, const uint32_t* count, uint32_t* part) {
+  dep_enter();
   uint32_t size = g->tbl_size;
   uint32_t base = blockIdx.x * kScanItems;
   if (base >= size) return;
@@ -271,6 +276,7 @@ __device__ __forceinline__ uint32_t block_incl_scan(uint32_t v, uint32_t* sh32) 
 
 // Single block: exclusive scan of the per-block partials (<= 4096 blocks).
 __global__ void k_scan_b(Grid* g, uint32_t* part) {
+  dep_enter();
   uint32_t nblk = (g->tbl_size + kScanItems - 1) / kScanItems;
   __shared__ uint32_t sh32[32];
   __shared__ uint32_t carry_s, carry_o;
@@ -302,6 +308,7 @@ __global__ void k_scan_b(Grid* g, uint32_t* part) {
 
 __global__ void k_scan_c(const Grid* g, const uint32_t* count, const uint32_t* part,
                          uint32_t* start, uint32_t* occ) {
+  dep_enter();
   uint32_t size = g->tbl_size;
   uint32_t base = blockIdx.x * kScanItems;
   if (base >= size) return;
@@ -330,6 +337,7 @@ __global__ void k_scan_c(const Grid* g, const uint32_t* count, const uint32_t* p
 
 __global__ void k_scatter(int64_t n, const uint32_t* code, const uint32_t* slot,
                           const uint32_t* start, int32_t* perm_tmp) {
+  dep_enter();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     perm_tmp[start[code[i]] + slot[i]] = (int32_t)i;
@@ -340,6 +348,7 @@ __global__ void k_scatter(int64_t n, const uint32_t* code, const uint32_t* slot,
 __global__ void k_cell_order(const Grid* g, const uint32_t* occ, const uint32_t* start,
                              const uint32_t* count, const int32_t* perm_tmp, int32_t* perm,
                              uint32_t* cell_of) {
+  dep_enter();
   const uint32_t n_occ = g->n_occ;
   const int lane = threadIdx.x & 31;
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
@@ -383,6 +392,7 @@ __device__ __forceinline__ uint32_t compact3(uint32_t v) {
 __global__ void k_gather_a(StateView in, StateView out, int64_t n, const double* org,
                            const int32_t* perm, const uint32_t* code, float4* pos32,
                            int32_t* cell3, float4* rec_d) {
+  dep_enter();
   constexpr int kRow = 1 << kMaxCellBits;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -416,6 +426,7 @@ __global__ void k_gather_a(StateView in, StateView out, int64_t n, const double*
 // search runs).  Loads before stores, as in k_gather_a.
 __global__ void k_gather_b(StateView in, StateView out, int64_t n, const int32_t* perm,
                            float4* rec_m, float4* recV) {
+  dep_enter();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int64_t s = p < n ? perm[p] : 0;
@@ -454,35 +465,34 @@ inline int grid_for(int64_t n, int threads, int sm) {
 void launch_grid(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st) {
   int blocks = grid_for(n, kRedThreads, ctx->sm_count);
   if (blocks > kReduceBlocks) blocks = kReduceBlocks;
-  k_grid_reduce<<<blocks, kRedThreads, 0, st>>>(in, n, ctx->prm, ctx->grid,
-                                                reinterpret_cast<long long*>(ctx->red.part),
-                                                ctx->red.counter + 0, ctx->err);
-  k_zero_table<<<ctx->sm_count * 8, 256, 0, st>>>(ctx->grid, ctx->tbl_count, ctx->cell_org);
+  launch_dep(k_grid_reduce, blocks, kRedThreads, 0, st, in, n, ctx->prm, ctx->grid,
+      reinterpret_cast<long long*>(ctx->red.part), ctx->red.counter + 0, ctx->err);
+  launch_dep(k_zero_table, ctx->sm_count * 8, 256, 0, st, ctx->grid, ctx->tbl_count, ctx->cell_org);
   ctx->launches += 2;
 }
 
 void launch_sort(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st,
                  cudaEvent_t wait_gather) {
   int pb = grid_for(n, 256, ctx->sm_count);
-  k_cell_count<<<pb, 256, 0, st>>>(in, n, ctx->grid, ctx->tbl_count, ctx->code, ctx->slot);
+  launch_dep(k_cell_count, pb, 256, 0, st, in, n, ctx->grid, ctx->tbl_count, ctx->code, ctx->slot);
   const int scan_blocks = kMaxTable / kScanItems;
-  k_scan_a<<<scan_blocks, kScanThreads, 0, st>>>(ctx->grid, ctx->tbl_count, ctx->scan_part);
-  k_scan_b<<<1, kScanThreads, 0, st>>>(ctx->grid, ctx->scan_part);
-  k_scan_c<<<scan_blocks, kScanThreads, 0, st>>>(ctx->grid, ctx->tbl_count, ctx->scan_part,
-                                                  ctx->tbl_start, ctx->occ);
-  k_scatter<<<pb, 256, 0, st>>>(n, ctx->code, ctx->slot, ctx->tbl_start, ctx->perm_tmp);
-  k_cell_order<<<ctx->sm_count * 8, 256, 0, st>>>(ctx->grid, ctx->occ, ctx->tbl_start,
-                                                  ctx->tbl_count, ctx->perm_tmp, ctx->perm,
-                                                  ctx->cell_of);
+  launch_dep(k_scan_a, scan_blocks, kScanThreads, 0, st, ctx->grid, ctx->tbl_count,
+      ctx->scan_part);
+  launch_dep(k_scan_b, 1, kScanThreads, 0, st, ctx->grid, ctx->scan_part);
+  launch_dep(k_scan_c, scan_blocks, kScanThreads, 0, st, ctx->grid, ctx->tbl_count,
+      ctx->scan_part, ctx->tbl_start, ctx->occ);
+  launch_dep(k_scatter, pb, 256, 0, st, n, ctx->code, ctx->slot, ctx->tbl_start, ctx->perm_tmp);
+  launch_dep(k_cell_order, ctx->sm_count * 8, 256, 0, st, ctx->grid, ctx->occ, ctx->tbl_start,
+      ctx->tbl_count, ctx->perm_tmp, ctx->perm, ctx->cell_of);
   if (wait_gather) cudaStreamWaitEvent(st, wait_gather, 0);
-  k_gather_a<<<pb, 256, 0, st>>>(in, ctx->s, n, ctx->cell_org, ctx->perm, ctx->code, ctx->pos32,
-                                 ctx->cell3, ctx->rec_d);
+  launch_dep(k_gather_a, pb, 256, 0, st, in, ctx->s, n, ctx->cell_org, ctx->perm, ctx->code,
+      ctx->pos32, ctx->cell3, ctx->rec_d);
   ctx->launches += 7;
 }
 
 void launch_gather_b(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st) {
-  k_gather_b<<<grid_for(n, 256, ctx->sm_count), 256, 0, st>>>(
-      in, ctx->s, n, ctx->perm, ctx->rec_m, staged_pairs(ctx) ? ctx->recV : nullptr);
+  launch_dep(k_gather_b, grid_for(n, 256, ctx->sm_count), 256, 0, st, in, ctx->s, n, ctx->perm,
+      ctx->rec_m, staged_pairs(ctx) ? ctx->recV : nullptr);
   ctx->launches += 1;
 }
 

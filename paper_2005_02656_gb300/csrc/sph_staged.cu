@@ -38,6 +38,7 @@
 #include "sph_device.cuh"
 #include "sph_find.cuh"
 #include "sph_internal.cuh"
+#include "sph_launch.cuh"
 #include "sph_tile.cuh"
 
 namespace sph {
@@ -422,6 +423,7 @@ __global__ void __launch_bounds__(kFindThreads, 4) k_find_mask(
     const Grid* gp, StateView s, const float4* __restrict__ pos32, const uint32_t* occ,
     const uint32_t* tbl_start, const uint32_t* tbl_count, int32_t* nn, uint32_t* nbr, int max_nb,
     MaskOut mo, uint32_t* err, unsigned long long* stats) {
+  dep_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   FindWarpSmem& W = reinterpret_cast<FindWarpSmem*>(smem_raw)[warp];
@@ -1131,6 +1133,7 @@ __device__ __forceinline__ void prefetch_cell(const Src& src, uint4 md,
 template <class Pass>
 __global__ void __launch_bounds__(kPT, Pass::kMinBlocks) k_cellpass(Pass pass, const Grid* gp,
                                                                     Src src) {
+  dep_enter();
   using SM = PassSmem<Pass>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* rec = reinterpret_cast<float4*>(smem_raw);
@@ -1345,6 +1348,7 @@ struct Share {
 template <class Pass>
 __global__ void __launch_bounds__(Pass::kPipeThreads, Pass::kPipeMinBlocks) k_cellpipe(
     Pass pass, const Grid* gp, PipeSrc src) {
+  dep_enter();
   using SM = PipeSmem<Pass>;
   constexpr int PT = SM::PT;
   constexpr int W = SM::W;
@@ -1657,8 +1661,8 @@ void launch_pass(sph_ctx* ctx, const Pass& p, int* cache, cudaStream_t st) {
   ps.nn = ctx->nn;
   ps.slist = reinterpret_cast<uint16_t*>(ctx->nbr);
   ps.max_nb = ctx->prm.max_nb;
-  k_cellpipe<Pass><<<pipe_blocks<Pass>(ctx, cache + 3), Pass::kPipeThreads,
-                     PipeSmem<Pass>::kBytes, st>>>(p, ctx->grid, ps);
+  launch_dep(k_cellpipe<Pass>, pipe_blocks<Pass>(ctx, cache + 3), Pass::kPipeThreads,
+      PipeSmem<Pass>::kBytes, st, p, ctx->grid, ps);
   // the general kernel: the other cells (for momentum also those of 449..832)
   Src src;
   src.meta = ctx->cmeta;
@@ -1669,13 +1673,13 @@ void launch_pass(sph_ctx* ctx, const Pass& p, int* cache, cudaStream_t st) {
   src.max_nb = ctx->prm.max_nb;
   src.cells = ctx->cells + ctx->n_max;
   src.ncells = ctx->salloc + 3;
-  k_cellpass<Pass><<<pass_blocks<Pass>(ctx, cache), kPT, PassSmem<Pass>::kBytes, st>>>(
-      p, ctx->grid, src);
+  launch_dep(k_cellpass<Pass>, pass_blocks<Pass>(ctx, cache), kPT, PassSmem<Pass>::kBytes, st, p,
+      ctx->grid, src);
   ctx->launches += 2;
   if (!Pass::kPipeAll) {
     src.cells = ctx->cells + 2 * ctx->n_max;
     src.ncells = ctx->salloc + 4;
-    k_cellpass<Pass><<<pass_blocks<Pass>(ctx, cache), kPT, PassSmem<Pass>::kBytes, st>>>(
+    launch_dep(k_cellpass<Pass>, pass_blocks<Pass>(ctx, cache), kPT, PassSmem<Pass>::kBytes, st,
         p, ctx->grid, src);
     ctx->launches += 1;
   }
@@ -1748,12 +1752,12 @@ void launch_find_masks(sph_ctx* ctx, const StateView& s, int64_t n, cudaStream_t
   mo.scells = ctx->cells + ctx->n_max;
   mo.mcells = ctx->cells + 2 * ctx->n_max;
   cudaMemsetAsync(ctx->salloc, 0, 5 * sizeof(unsigned long long), st);
-  k_find_mask<false><<<ctx->find_mask_blocks, kFindThreads, smem, st>>>(
-      ctx->grid, s, ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr,
-      ctx->prm.max_nb, mo, ctx->err, ctx->stats);
-  k_find_mask<true><<<ctx->find_mask_blocks, kFindThreads, smem, st>>>(
-      ctx->grid, s, ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr,
-      ctx->prm.max_nb, mo, ctx->err, ctx->stats);
+  launch_dep(k_find_mask<false>, ctx->find_mask_blocks, kFindThreads, smem, st, ctx->grid, s,
+      ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb,
+      mo, ctx->err, ctx->stats);
+  launch_dep(k_find_mask<true>, ctx->find_mask_blocks, kFindThreads, smem, st, ctx->grid, s,
+      ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb,
+      mo, ctx->err, ctx->stats);
   ctx->launches += 2;
 }
 

@@ -21,6 +21,7 @@
 
 #include "sph_device.cuh"
 #include "sph_internal.cuh"
+#include "sph_launch.cuh"
 
 namespace sph {
 
@@ -120,6 +121,7 @@ __global__ void __launch_bounds__(kThreads) k_timestep(const double* h, const do
                                                        double energy_dt, double* dt_io,
                                                        double* diag, double* part,
                                                        unsigned int* counter, uint32_t* err) {
+  dep_enter();
   double mn = INFINITY, mu = INFINITY;
   float lim = INFINITY;  // FP32 screen value of mn
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -205,6 +207,7 @@ __global__ void __launch_bounds__(kThreads) k_update(StateView s, OutView o, Sta
                                                      double* diag, double* part,
                                                      unsigned int* counter,
                                                      unsigned long long* stats) {
+  dep_enter();
   const double dt = diag[8], dt_prev = diag[12];
   const double delta = 0.5 * (dt + dt_prev);
   const double q = dt_prev > 0.0 ? dt / (2.0 * dt_prev) : 0.0;
@@ -364,9 +367,9 @@ inline int red_blocks(int64_t n, int sm) {
 
 void launch_timestep(sph_ctx* ctx, const StateView& s, const OutView& o, int64_t n, double* dt_io,
                      cudaStream_t st) {
-  k_timestep<<<red_blocks(n, ctx->sm_count), kThreads, 0, st>>>(
-      s.h, o.c, s.u, o.du, n, ctx->prm.courant, ctx->prm.dt_growth, ctx->prm.energy_dt, dt_io,
-      ctx->diag, ctx->red.part, ctx->red.counter + 1, ctx->err);
+  launch_dep(k_timestep, red_blocks(n, ctx->sm_count), kThreads, 0, st, s.h, o.c, s.u, o.du, n,
+      ctx->prm.courant, ctx->prm.dt_growth, ctx->prm.energy_dt, dt_io, ctx->diag, ctx->red.part,
+      ctx->red.counter + 1, ctx->err);
   ctx->launches += 1;
 }
 
@@ -381,9 +384,8 @@ void launch_update(sph_ctx* ctx, const StateView& s, const OutView& o, const Sta
   (void)dt_io;
   if (ctx->hfac_ng != ctx->prm.ng_target) launch_hfac_table(ctx, st);
   auto kern = ctx->prm.angular_sums ? k_update<true> : k_update<false>;
-  kern<<<red_blocks(n, ctx->sm_count), kThreads, 0, st>>>(
-      s, o, dst, ctx->nn, n, ctx->prm, ctx->hfac, ctx->diag, ctx->red.part,
-      ctx->red.counter + 2, ctx->stats);
+  launch_dep(kern, red_blocks(n, ctx->sm_count), kThreads, 0, st, s, o, dst, ctx->nn, n, ctx->prm,
+      ctx->hfac, ctx->diag, ctx->red.part, ctx->red.counter + 2, ctx->stats);
   ctx->launches += 1;
 }
 
