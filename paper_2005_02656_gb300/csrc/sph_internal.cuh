@@ -11,7 +11,7 @@ namespace sph {
 
 constexpr int kMaxCellBits = 8;                 // up to 256 cells per axis
 constexpr uint32_t kMaxTable = 1u << (3 * kMaxCellBits);
-constexpr int kReduceBlocks = 1024;             // partial slots of grid reductions
+constexpr int kReduceBlocks = 2048;             // partial slots of grid reductions
 constexpr int kScanItems = 4096;                // cell-table entries per scan block
 constexpr int kProfRing = 64;                   // step event sets kept before folding
 constexpr int kHTab = 4097;                     // h factors tabulated for counts 0..4096
@@ -146,9 +146,9 @@ struct sph_ctx {
   float4* recC;
   float2* recC2;
   int find_mask_blocks;   // persistent CTAs of the mask-writing search
-  int pass_blocks[12];    // persistent CTAs of the density, IAD, momentum passes (general
-                          // kernels, then pipelined ones at +3; the plain-configuration
-                          // kernels at +6)
+  int pass_blocks[2][3][3];  // persistent CTAs of the pair passes: general or plain
+                             // configuration; density, IAD, momentum; both forms in one
+                             // launch, pipelined form, general form
 
   // reductions
   sph::Reduce red;

@@ -18,12 +18,9 @@ namespace {
 
 using namespace find;
 
-// Launched in both variants; the one whose WRAP does not match the grid (a
-// periodic axis with fewer than 3 cells needs the FP32 wrap) returns at once.
 // No register cap: at 108-122 registers (4 CTAs per SM) the search measured
 // 1-2% faster than capped at 94 (5 CTAs) or 80 (6 CTAs); its unrolled mask
 // loop gains more from registers than from resident warps.
-template <bool WRAP>
 __global__ void __launch_bounds__(kFindThreads, 1) k_find_tile(
     const Grid* gp, StateView s, const float4* __restrict__ pos32, const uint32_t* occ,
     const uint32_t* tbl_start, const uint32_t* tbl_count, int32_t* nn, uint32_t* nbr,
@@ -33,12 +30,17 @@ __global__ void __launch_bounds__(kFindThreads, 1) k_find_tile(
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   FindWarpSmem& W = reinterpret_cast<FindWarpSmem*>(smem_raw)[warp];
   const Grid g = *gp;
-  if ((g.wrap32 != 0) != WRAP) return;
   unsigned long long tested = 0, exact = 0;
   const uint32_t gw = blockIdx.x * kFindWarps + warp, nw = gridDim.x * kFindWarps;
-  for (uint32_t cell = gw; cell < g.n_occ; cell += nw)
-    find_cell<WRAP>(g, occ[cell], s, pos32, tbl_start, tbl_count, nn, nbr, max_nb, err, W,
-                    tested, exact);
+  if (g.wrap32) {  // a periodic axis with fewer than 3 cells: FP32 separations need the wrap
+    for (uint32_t cell = gw; cell < g.n_occ; cell += nw)
+      find_cell<true>(g, occ[cell], s, pos32, tbl_start, tbl_count, nn, nbr, max_nb, err, W,
+                      tested, exact);
+  } else {
+    for (uint32_t cell = gw; cell < g.n_occ; cell += nw)
+      find_cell<false>(g, occ[cell], s, pos32, tbl_start, tbl_count, nn, nbr, max_nb, err, W,
+                       tested, exact);
+  }
   // counters: one atomic per warp
   for (int o = 16; o > 0; o >>= 1) {
     tested += __shfl_xor_sync(0xffffffffu, tested, o);
@@ -78,21 +80,15 @@ void launch_find_neighbors(sph_ctx* ctx, const StateView& s, int64_t n, cudaStre
   const size_t smem = kFindWarps * sizeof(FindWarpSmem);
   if (!ctx->find_blocks) {  // once per context, on its device
     int per_sm = 0;
-    cudaFuncSetAttribute(k_find_tile<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    cudaFuncSetAttribute(k_find_tile<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_find_tile<false>, kFindThreads,
+    cudaFuncSetAttribute(k_find_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_find_tile, kFindThreads,
                                                   smem);
     ctx->find_blocks = (per_sm > 0 ? per_sm : 1) * ctx->sm_count;
   }
-  launch_dep(k_find_tile<false>, ctx->find_blocks, kFindThreads, smem, st, ctx->grid, s,
-      ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb,
-      ctx->err, ctx->stats);
-  launch_dep(k_find_tile<true>, ctx->find_blocks, kFindThreads, smem, st, ctx->grid, s, ctx->pos32,
-      ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb, ctx->err,
-      ctx->stats);
-  ctx->launches += 2;
+  launch_dep(k_find_tile, ctx->find_blocks, kFindThreads, smem, st, ctx->grid, s, ctx->pos32,
+             ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb, ctx->err,
+             ctx->stats);
+  ctx->launches += 1;
 }
 
 void launch_export_neighbors(sph_ctx* ctx, const StateView& s, int64_t n, int32_t* counts,

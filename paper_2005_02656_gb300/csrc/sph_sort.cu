@@ -99,19 +99,19 @@ __global__ void k_grid_reduce(StateView in, int64_t n, sph_params prm, Grid* g, 
   if (l == 0)
     for (int k = 0; k < 7; ++k) sh[w][k] = r[k];
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int ww = 1; ww < (int)(blockDim.x >> 5); ++ww) {
-    for (int k = 0; k < 3; ++k) r[k] = min(r[k], sh[ww][k]);
-    for (int k = 3; k < 7; ++k) r[k] = max(r[k], sh[ww][k]);
+  // the grid: thread ax derives axis ax (the divisions of the three side by side)
+  __shared__ Grid G;
+  if (threadIdx.x < 7) {
+    const int k = threadIdx.x;
+    long long q = sh[0][k];
+    for (int ww = 1; ww < (int)(blockDim.x >> 5); ++ww)
+      q = k < 3 ? min(q, sh[ww][k]) : max(q, sh[ww][k]);
+    sh[0][k] = q;
   }
-  double rd[7];
-  for (int k = 0; k < 7; ++k) rd[k] = from_okey(r[k]);
-  *counter = 0;
-  Grid G;
-  double hmax = rd[6];
-  G.hmax = hmax;
-  int maxnc = 1;
-  for (int ax = 0; ax < 3; ++ax) {
+  __syncthreads();
+  const double hmax = from_okey(sh[0][6]);
+  if (threadIdx.x < 3) {
+    const int ax = threadIdx.x;
     int per = prm.periodic[ax] ? 1 : 0;
     double lo, L;
     if (per) {
@@ -119,8 +119,8 @@ __global__ void k_grid_reduce(StateView in, int64_t n, sph_params prm, Grid* g, 
       L = prm.box_hi[ax] - prm.box_lo[ax];
       if (!(2.0 * hmax < 0.5 * L)) raise_flag(err, SPH_FLAG_BAD_BOX);
     } else {
-      lo = n > 0 ? rd[ax] : 0.0;
-      L = n > 0 ? rd[3 + ax] - rd[ax] : 0.0;
+      lo = n > 0 ? from_okey(sh[0][ax]) : 0.0;
+      L = n > 0 ? from_okey(sh[0][3 + ax]) - from_okey(sh[0][ax]) : 0.0;
     }
     int nc = 1;
     if (hmax > 0.0 && L > 0.0) {
@@ -139,11 +139,17 @@ __global__ void k_grid_reduce(StateView in, int64_t n, sph_params prm, Grid* g, 
     G.err32[ax] = (float)(cs * 9.5367431640625e-07);  // 2^-20 cs
     G.nc[ax] = nc;
     G.periodic[ax] = per;
-    maxnc = nc > maxnc ? nc : maxnc;
   }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  *counter = 0;
+  G.hmax = hmax;
   G.wrap32 = 0;
-  for (int ax = 0; ax < 3; ++ax)
+  int maxnc = 1;
+  for (int ax = 0; ax < 3; ++ax) {
+    maxnc = max(maxnc, G.nc[ax]);
     if (G.periodic[ax] && G.nc[ax] < 3) G.wrap32 = 1;
+  }
   int bits = 0;
   while ((1 << bits) < maxnc) ++bits;
   G.bits = bits;
@@ -218,36 +224,35 @@ constexpr int kPerThread = kScanItems / kScanThreads;
 
 __global__ void k_scan_a(const Grid* g, const uint32_t* count, uint32_t* part) {
   dep_enter();
-  uint32_t size = g->tbl_size;
-  uint32_t base = blockIdx.x * kScanItems;
-  if (base >= size) return;
-  uint32_t s = 0, o = 0;
-  for (int k = 0; k < kPerThread; ++k) {
-    uint32_t i = base + threadIdx.x * kPerThread + k;
-    if (i < size) {
-      uint32_t c = count[i];
-      s += c;
-      o += c ? 1u : 0u;
-    }
-  }
-  for (int off = 16; off > 0; off >>= 1) {
-    s += __shfl_xor_sync(0xffffffffu, s, off);
-    o += __shfl_xor_sync(0xffffffffu, o, off);
-  }
+  const uint32_t size = g->tbl_size;
   __shared__ uint32_t ss[32], so[32];
-  if ((threadIdx.x & 31) == 0) {
-    ss[threadIdx.x >> 5] = s;
-    so[threadIdx.x >> 5] = o;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t ts = 0, to = 0;
-    for (int w = 0; w < kScanThreads / 32; ++w) {
-      ts += ss[w];
-      to += so[w];
+  for (uint32_t blk = blockIdx.x; blk * kScanItems < size; blk += gridDim.x) {
+    const uint32_t base = blk * kScanItems;
+    uint32_t s = 0, o = 0;
+    for (int k = 0; k < kPerThread; ++k) {
+      uint32_t i = base + threadIdx.x * kPerThread + k;
+      if (i < size) {
+        uint32_t c = count[i];
+        s += c;
+        o += c ? 1u : 0u;
+      }
     }
-    part[2 * blockIdx.x] = ts;
-    part[2 * blockIdx.x + 1] = to;
+    s = __reduce_add_sync(0xffffffffu, s);
+    o = __reduce_add_sync(0xffffffffu, o);
+    if ((threadIdx.x & 31) == 0) {
+      ss[threadIdx.x >> 5] = s;
+      so[threadIdx.x >> 5] = o;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const uint32_t ts = __reduce_add_sync(0xffffffffu, ss[threadIdx.x]);
+      const uint32_t to = __reduce_add_sync(0xffffffffu, so[threadIdx.x]);
+      if (threadIdx.x == 0) {
+        part[2 * blk] = ts;
+        part[2 * blk + 1] = to;
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -309,28 +314,29 @@ __global__ void k_scan_b(Grid* g, uint32_t* part) {
 __global__ void k_scan_c(const Grid* g, const uint32_t* count, const uint32_t* part,
                          uint32_t* start, uint32_t* occ) {
   dep_enter();
-  uint32_t size = g->tbl_size;
-  uint32_t base = blockIdx.x * kScanItems;
-  if (base >= size) return;
+  const uint32_t size = g->tbl_size;
   __shared__ uint32_t sh32[32];
-  uint32_t c[kPerThread];
-  uint32_t s = 0, o = 0;
-  for (int k = 0; k < kPerThread; ++k) {
-    uint32_t i = base + threadIdx.x * kPerThread + k;
-    c[k] = i < size ? count[i] : 0u;
-    s += c[k];
-    o += c[k] ? 1u : 0u;
-  }
-  uint32_t is = block_incl_scan(s, sh32);
-  uint32_t io = block_incl_scan(o, sh32);
-  uint32_t ps = part[2 * blockIdx.x] + is - s;
-  uint32_t po = part[2 * blockIdx.x + 1] + io - o;
-  for (int k = 0; k < kPerThread; ++k) {
-    uint32_t i = base + threadIdx.x * kPerThread + k;
-    if (i < size) {
-      start[i] = ps;
-      if (c[k]) occ[po++] = i;
-      ps += c[k];
+  for (uint32_t blk = blockIdx.x; blk * kScanItems < size; blk += gridDim.x) {
+    const uint32_t base = blk * kScanItems;
+    uint32_t c[kPerThread];
+    uint32_t s = 0, o = 0;
+    for (int k = 0; k < kPerThread; ++k) {
+      uint32_t i = base + threadIdx.x * kPerThread + k;
+      c[k] = i < size ? count[i] : 0u;
+      s += c[k];
+      o += c[k] ? 1u : 0u;
+    }
+    uint32_t is = block_incl_scan(s, sh32);
+    uint32_t io = block_incl_scan(o, sh32);
+    uint32_t ps = part[2 * blk] + is - s;
+    uint32_t po = part[2 * blk + 1] + io - o;
+    for (int k = 0; k < kPerThread; ++k) {
+      uint32_t i = base + threadIdx.x * kPerThread + k;
+      if (i < size) {
+        start[i] = ps;
+        if (c[k]) occ[po++] = i;
+        ps += c[k];
+      }
     }
   }
 }
@@ -475,7 +481,9 @@ void launch_sort(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st,
                  cudaEvent_t wait_gather) {
   int pb = grid_for(n, 256, ctx->sm_count);
   launch_dep(k_cell_count, pb, 256, 0, st, in, n, ctx->grid, ctx->tbl_count, ctx->code, ctx->slot);
-  const int scan_blocks = kMaxTable / kScanItems;
+  // as many blocks as run at once, not one per chunk of the largest table
+  // (4,096, most of which a smaller grid leaves at once: 10 + 7 us of a small step)
+  const int scan_blocks = 2 * ctx->sm_count;
   launch_dep(k_scan_a, scan_blocks, kScanThreads, 0, st, ctx->grid, ctx->tbl_count,
       ctx->scan_part);
   launch_dep(k_scan_b, 1, kScanThreads, 0, st, ctx->grid, ctx->scan_part);

@@ -22,7 +22,7 @@
 // (upper bounds: the stencil's particle count P for the entries, na ceil(P/64)
 // for the masks), so the layout depends on scheduling but the contents do not.
 //
-// Pair passes (k_cellpass, one CTA of kPT threads per occupied cell at a time).
+// Pair passes (one CTA of kPT threads per occupied cell at a time).
 // The cell's staged candidate records are copied once into shared memory,
 // with their cell shift applied, so separations are FP32 differences of
 // positions relative to the target cell.  Each target's staged-slot list
@@ -144,7 +144,16 @@ __device__ __forceinline__ int write_slot_list(const unsigned long long* words, 
   return k;
 }
 
-template <bool WRAP, int WIN>
+// PARTS = 1: one warp takes the whole cell.  PARTS = kFindWarps: the warps of a
+// CTA take a quarter of its targets each, all staging the candidates for
+// themselves; warp 0 also writes what belongs to the cell (`sh` carries its
+// allocation, and back the largest hit count).
+struct PartShared {
+  unsigned long long sb, mb;
+  int kmax;
+};
+
+template <bool WRAP, int WIN, int PARTS>
 __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, uint32_t code,
                                                 const StateView& s,
                                                 const float4* __restrict__ pos32,
@@ -156,8 +165,10 @@ __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, ui
                                                 unsigned long long& exact,
                                                 unsigned long long& slots,
                                                 unsigned long long& words,
-                                                unsigned long long* mbuf) {
+                                                unsigned long long* mbuf, PartShared* sh) {
   const int lane = threadIdx.x & 31;
+  const int part = PARTS > 1 ? (int)(threadIdx.x >> 5) : 0;
+  const bool lead_warp = part == 0;
   Stencil& S = W.S;
   const float esum = g.err32[0] + g.err32[1] + g.err32[2];
   const float esq = g.err32[0] * g.err32[0] + g.err32[1] * g.err32[1] + g.err32[2] * g.err32[2];
@@ -168,12 +179,23 @@ __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, ui
   unsigned long long sb = 0, mb = 0;
   if (ok) {
     const unsigned long long nblk_max = (unsigned long long)((P + 63) >> 6);
-    if (lane == 0) {
+    if (lane == 0 && lead_warp) {
       sb = atomicAdd(mo.alloc + 0, (unsigned long long)P);
       mb = atomicAdd(mo.alloc + 1, (unsigned long long)na * nblk_max);
     }
-    sb = __shfl_sync(0xffffffffu, sb, 0);
-    mb = __shfl_sync(0xffffffffu, mb, 0);
+    if (PARTS > 1) {
+      if (threadIdx.x == 0) {
+        sh->sb = sb;
+        sh->mb = mb;
+        sh->kmax = 0;
+      }
+      __syncthreads();
+      sb = sh->sb;
+      mb = sh->mb;
+    } else {
+      sb = __shfl_sync(0xffffffffu, sb, 0);
+      mb = __shfl_sync(0xffffffffu, mb, 0);
+    }
     // cannot fail (sum of P <= 27 n, sum of na ceil(P/64) <= kMaskWords n); kept
     // as a guard
     ok = sb + (unsigned long long)P <= mo.sent_cap &&
@@ -182,9 +204,10 @@ __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, ui
   if (!ok) {
     // list form: the list-writing search of sph_find.cuh for this cell
     __syncwarp();
-    find::find_cell<WRAP, WIN>(g, code, s, pos32, tbl_start, tbl_count, nn, nbr, max_nb, err,
-                               W, tested, exact);
-    if (lane == 0) {
+    if (lead_warp)
+      find::find_cell<WRAP, WIN>(g, code, s, pos32, tbl_start, tbl_count, nn, nbr, max_nb, err,
+                                 W, tested, exact);
+    if (lane == 0 && lead_warp) {
       mo.meta[cell] = make_uint4(0u, kListForm, (uint32_t)a0, (uint32_t)na & 0xffffu);
       mo.scells[atomicAdd(mo.alloc + 3, 1ull)] = cell;
     }
@@ -234,6 +257,7 @@ __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, ui
   // in the warp's mask buffer (word jb of lane t at mbuf[32 jb + t]) and the
   // round's lists are written from there, so its masks never reach memory.
   bool direct = false;
+  const int t_lo = na * part / PARTS, t_hi = na * (part + 1) / PARTS;
   int kmax = 0;        // largest hit count of the cell's targets (direct cells)
   int sc = 0, j0 = 0;  // next source: stencil cell and particle within it
   const uint32_t lt = (1u << lane) - 1u;
@@ -277,7 +301,7 @@ __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, ui
           W.cz[pq] = cz;
           const uint32_t e = ecode | (uint32_t)(st + j);
           W.entry[q] = e;
-          mo.sent[slot_base + 64u * gb + (uint32_t)q] = e;
+          if (lead_warp) mo.sent[slot_base + 64u * gb + (uint32_t)q] = e;
         }
         wn += __popc(bal);
         j0 += 32;
@@ -301,11 +325,11 @@ __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, ui
     __syncwarp();
     const int nproc = done ? wn : 64 * nblk;  // real slots processed now
     direct = first && done;
-    for (int t0 = 0; t0 < na; t0 += 32) {
+    for (int t0 = t_lo; t0 < t_hi; t0 += 32) {
       // a round of r targets; with r <= 16, G = 32 / r lanes share each target
       // and take its blocks round-robin (lane l: target l % r, blocks
       // jb = l / r, l / r + G, ...)
-      const int r = min(32, na - t0);
+      const int r = min(32, t_hi - t0);
       const int G = 32 / r;
       const int tl = lane % r, grp = lane / r;
       const bool active = grp < G;
@@ -376,7 +400,7 @@ __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, ui
     __syncwarp();
   }
   const uint32_t staged = 64u * gb + (uint32_t)wn;
-  if (lane == 0) {
+  if (lane == 0 && lead_warp) {
     slots += staged;
     words += (unsigned long long)na * ((staged + 63) >> 6);
   }
@@ -390,25 +414,30 @@ __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, ui
   static_assert(kStagedMaxP / 64 * 32 * 8 <= 4 * WIN * 4, "mask copy fits the window");
   unsigned long long* mcopy = reinterpret_cast<unsigned long long*>(W.cx);
   int kl = 0;  // this lane's count
-  for (int t0 = 0; !direct && t0 < na; t0 += 32, kmax = max(kmax, kl), kl = 0) {
+  for (int t0 = t_lo; !direct && t0 < t_hi; t0 += 32, kmax = max(kmax, kl), kl = 0) {
     const int t = t0 + lane;
     __syncwarp();
 #pragma unroll 4
     for (int blk = 0; blk < nblk; ++blk)
       mcopy[blk * 32 + lane] =
-          t < na ? mo.masks[mask_base + (uint32_t)blk * (uint32_t)na + (uint32_t)t] : 0ull;
+          t < t_hi ? mo.masks[mask_base + (uint32_t)blk * (uint32_t)na + (uint32_t)t] : 0ull;
     __syncwarp();
-    if (t >= na) continue;
+    if (t >= t_hi) continue;
     kl = write_slot_list(mcopy + lane, nblk, slot_row(mo.slist, (int64_t)a0 + t, max_nb), max_nb);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
+  if (PARTS > 1) {
+    if (lane == 0) atomicMax(&sh->kmax, kmax);
+    __syncthreads();
+    kmax = sh->kmax;
+  }
   // cells the pipelined passes take whole: one round of at most kTR targets,
   // lists of at most kLC entries and one window of staged candidates (448
   // for momentum, 832 for the others)
   const int cls =
       na > kTR || kmax > kLC || (int)staged > kPipeWin ? 1 : ((int)staged <= kPipeWinM ? 0 : 2);
-  if (lane == 0) {
+  if (lane == 0 && lead_warp) {
     mo.meta[cell] = make_uint4(slot_base, (uint32_t)gself, (uint32_t)a0,
                                (staged << 16) | (cls != 1 ? 0x8000u : 0u) | (uint32_t)na);
     const unsigned long long q = atomicAdd(mo.alloc + 2 + cls, 1ull);
@@ -435,8 +464,9 @@ __global__ void __launch_bounds__(kFindThreads, 4) k_find_mask(
   unsigned long long tested = 0, exact = 0, slots = 0, words = 0;
   const uint32_t gw = blockIdx.x * kFindWarps + warp, nw = gridDim.x * kFindWarps;
   for (uint32_t cell = gw; cell < g.n_occ; cell += nw)
-    find_cell_masks<WRAP, kFindWindow>(g, cell, occ[cell], s, pos32, tbl_start, tbl_count, nn,
-                                       nbr, max_nb, mo, err, W, tested, exact, slots, words, mbuf);
+    find_cell_masks<WRAP, kFindWindow, 1>(g, cell, occ[cell], s, pos32, tbl_start, tbl_count, nn,
+                                          nbr, max_nb, mo, err, W, tested, exact, slots, words,
+                                          mbuf, nullptr);
   for (int o = 16; o > 0; o >>= 1) {
     tested += __shfl_xor_sync(0xffffffffu, tested, o);
     exact += __shfl_xor_sync(0xffffffffu, exact, o);
@@ -449,9 +479,46 @@ __global__ void __launch_bounds__(kFindThreads, 4) k_find_mask(
   }
 }
 
+// The same by one CTA per cell, for states with too few cells to give every
+// warp one (launch_find_masks).
+template <bool WRAP>
+__global__ void __launch_bounds__(kFindThreads, 4) k_find_mask_cta(
+    const Grid* gp, StateView s, const float4* __restrict__ pos32, const uint32_t* occ,
+    const uint32_t* tbl_start, const uint32_t* tbl_count, int32_t* nn, uint32_t* nbr, int max_nb,
+    MaskOut mo, uint32_t* err, unsigned long long* stats) {
+  dep_enter();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ PartShared sh;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  FindWarpSmem& W = reinterpret_cast<FindWarpSmem*>(smem_raw)[warp];
+  unsigned long long* mbuf = reinterpret_cast<unsigned long long*>(
+                                 smem_raw + kFindWarps * sizeof(FindWarpSmem)) +
+                             warp * kMaskBufWords;
+  const Grid g = *gp;
+  if ((g.wrap32 != 0) != WRAP) return;
+  unsigned long long tested = 0, exact = 0, slots = 0, words = 0;
+  for (uint32_t cell = blockIdx.x; cell < g.n_occ; cell += gridDim.x) {
+    find_cell_masks<WRAP, kFindWindow, kFindWarps>(g, cell, occ[cell], s, pos32, tbl_start,
+                                                   tbl_count, nn, nbr, max_nb, mo, err, W, tested,
+                                                   exact, slots, words, mbuf, &sh);
+    __syncthreads();  // sh is free for the next cell
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    tested += __shfl_xor_sync(0xffffffffu, tested, o);
+    exact += __shfl_xor_sync(0xffffffffu, exact, o);
+  }
+  if (lane == 0) {
+    atomicAdd(stats + 0, tested);
+    atomicAdd(stats + 1, exact);
+    atomicAdd(stats + 4, slots);
+    atomicAdd(stats + 5, words);
+  }
+}
+
 // ------------------------------------------------------------- pair passes --
 
-constexpr int kPT = 256;        // threads per CTA (general pair passes)
+constexpr int kPT = 256;        // threads per CTA of the pair passes
+constexpr int kPassBlocks = 3;  // CTAs per SM
 constexpr int kLS = kLC + 8;    // list row stride (uint16): 16-byte aligned rows, in different banks
 constexpr int kMaxSub = 32;     // threads sharing one target, at most
 
@@ -569,10 +636,8 @@ struct DensityPassT {
   static constexpr int kWin = 1024;   // staged slots held in shared memory
   static constexpr int kRecBytes = 16;
   static constexpr int kV = 2;        // reduced values: sum m S^n, grad-h sum
-  static constexpr int kMinBlocks = 4;
   static constexpr bool kPaired = true;  // two pairs per iteration in paired FP32
   static constexpr int kPipeThreads = 256;
-  static constexpr int kPipeMinBlocks = 3;
   static constexpr int kPipeW = kPipeWin;  // its window (staged slots per buffer)
   static constexpr bool kPipeAll = true;   // cells of up to kPipeWin candidates
   static constexpr bool kSmemLists = true; // lists copied with the records
@@ -698,11 +763,8 @@ struct IadPassT {
   static constexpr int kWin = 1024;
   static constexpr int kRecBytes = 16;
   static constexpr int kV = 6;
-  static constexpr int kMinBlocks = 3;  // general kernel (the few cells outside the pipelined
-                                        // lists): no register spills at this bound
   static constexpr bool kPaired = true;
   static constexpr int kPipeThreads = 256;
-  static constexpr int kPipeMinBlocks = 3;
   static constexpr int kPipeW = kPipeWin;
   static constexpr bool kPipeAll = true;
   static constexpr bool kSmemLists = true;
@@ -841,13 +903,11 @@ struct MomentumPassT {
   // formed per record read): 8 bytes fewer per pair from shared memory
   static constexpr int kRecBytes = CFG == kCfgPlain ? 64 : 72;
   static constexpr int kV = 4;
-  static constexpr int kMinBlocks = 3;
   static constexpr bool kPaired = false;  // the paired body needs ~120 registers: scalar pairs
                                           // keep three CTAs per SM
   // pipelined kernel: cells of up to kPipeWinM candidates, a double buffer of
   // 2 x 32 KB, three CTAs per SM
   static constexpr int kPipeThreads = 256;
-  static constexpr int kPipeMinBlocks = 3;
   static constexpr int kPipeW = kPipeWinM;
   static constexpr bool kPipeAll = false;    // the cells of 449..832 candidates: general kernel
   static constexpr bool kSmemLists = false;  // lists read through L1
@@ -1093,6 +1153,8 @@ struct Src {
   const uint4* meta;                 // per occupied cell
   const uint32_t* cells;             // the cells of this launch
   const unsigned long long* ncells;  // their number (device counter)
+  const uint32_t* cells1;            // a second list (may be null)
+  const unsigned long long* ncells1;
   const uint32_t* sent;              // staged candidate entries
   const int32_t* nn;                 // exact neighbour counts
   const uint32_t* nbr;               // list-form cells: int32 lists
@@ -1130,34 +1192,34 @@ __device__ __forceinline__ void prefetch_cell(const Src& src, uint4 md,
   }
 }
 
+// The general form, by CTA `blk` of G.
 template <class Pass>
-__global__ void __launch_bounds__(kPT, Pass::kMinBlocks) k_cellpass(Pass pass, const Grid* gp,
-                                                                    Src src) {
-  dep_enter();
+__device__ __forceinline__ void cellpass(const Pass& pass, const Grid* gp, const Src& src,
+                                         const uint32_t* cells, const unsigned long long* ncells,
+                                         uint32_t blk, uint32_t G) {
+  const uint32_t n_cells = (uint32_t)*ncells;
+  if (blk >= n_cells) return;
+  const Grid g = *gp;
   using SM = PassSmem<Pass>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* rec = reinterpret_cast<float4*>(smem_raw);
   uint16_t* lists = reinterpret_cast<uint16_t*>(smem_raw + SM::kRec);
   float* part = reinterpret_cast<float*>(smem_raw + SM::kRec);
   int* tot = reinterpret_cast<int*>(smem_raw + SM::oTot);
-  const Grid g = *gp;
-  if (!pass.runs(g)) return;
   Tabs tb(smem_raw + SM::oTab);
   tb.fill<kPT>(g);
-  const uint32_t n_cells = (uint32_t)*src.ncells;
-  const uint32_t G = gridDim.x;
   const int tid = threadIdx.x;
   const uint4 zero4 = make_uint4(0u, kListForm, 0u, 0u);
-  auto meta_of = [&](uint32_t q) { return q < n_cells ? __ldg(src.meta + src.cells[q]) : zero4; };
-  auto cell_at = [&](uint32_t q) { return q < n_cells ? __ldg(src.cells + q) : kNoCell; };
+  auto meta_of = [&](uint32_t q) { return q < n_cells ? __ldg(src.meta + cells[q]) : zero4; };
+  auto cell_at = [&](uint32_t q) { return q < n_cells ? __ldg(cells + q) : kNoCell; };
   auto meta_at = [&](uint32_t c) { return c != kNoCell ? __ldg(src.meta + c) : zero4; };
-  uint4 md_next = meta_of(blockIdx.x);
-  uint4 md_after = meta_of(blockIdx.x + G);
-  uint32_t c_ahead = cell_at(blockIdx.x + 2 * G);  // meta loaded one cell later
+  uint4 md_next = meta_of(blk);
+  uint4 md_after = meta_of(blk + G);
+  uint32_t c_ahead = cell_at(blk + 2 * G);  // meta loaded one cell later
   constexpr int NJ = window_slots<Pass>();
   Prefetch<NJ> pf;
   prefetch_cell<Pass>(src, md_next, pf);
-  for (uint32_t q = blockIdx.x; q < n_cells; q += G) {
+  for (uint32_t q = blk; q < n_cells; q += G) {
     const uint4 md = md_next;
     const Prefetch<NJ> cur = pf;
     md_next = md_after;
@@ -1346,9 +1408,8 @@ struct Share {
 
 
 template <class Pass>
-__global__ void __launch_bounds__(Pass::kPipeThreads, Pass::kPipeMinBlocks) k_cellpipe(
-    Pass pass, const Grid* gp, PipeSrc src) {
-  dep_enter();
+__device__ __forceinline__ void cellpipe(const Pass& pass, const Grid* gp, const PipeSrc& src,
+                                         uint32_t blk, uint32_t G) {
   using SM = PipeSmem<Pass>;
   constexpr int PT = SM::PT;
   constexpr int W = SM::W;
@@ -1364,17 +1425,15 @@ __global__ void __launch_bounds__(Pass::kPipeThreads, Pass::kPipeMinBlocks) k_ce
   auto part = [&](int h) {
     return reinterpret_cast<float*>(smem_raw + SM::oPart + h * SM::kPart);
   };
+  const uint32_t n0 = (uint32_t)*src.n0;
+  const uint32_t n_cells = n0 + (src.cells1 ? (uint32_t)*src.n1 : 0u);
+  uint32_t q = blk;
+  if (q >= n_cells) return;
   const Grid g = *gp;
-  if (!pass.runs(g)) return;
   const int tid = threadIdx.x;
   Tabs tb(smem_raw + SM::oTab);
   tb.fill<PT>(g);
   const float4* shtab = tb.shift;
-  const uint32_t n0 = (uint32_t)*src.n0;
-  const uint32_t n_cells = n0 + (src.cells1 ? (uint32_t)*src.n1 : 0u);
-  const uint32_t G = gridDim.x;
-  uint32_t q = blockIdx.x;
-  if (q >= n_cells) return;
   const uint4 none = make_uint4(0u, kListForm, 0u, 0u);
   auto cell_at = [&](uint32_t qq) {
     return qq < n0 ? __ldg(src.cells0 + qq)
@@ -1616,73 +1675,121 @@ __global__ void __launch_bounds__(Pass::kPipeThreads, Pass::kPipeMinBlocks) k_ce
   }
 }
 
+// One launch of a pass: its first `half` CTAs run the pipelined form over
+// their cells, the other `half` the general form over the others (for momentum
+// first those of 449..832 candidates, then the rest).  On a small state the two
+// run side by side; on a large one the others start as the first run out
+// of cells.
 template <class Pass>
-int pipe_blocks(sph_ctx* ctx, int* cache) {
+__device__ __forceinline__ void run_pass(const Pass& pass, const Grid* gp, const PipeSrc& ps,
+                                         const Src& src, uint32_t half) {
+  static_assert(Pass::kPipeThreads == kPT, "one CTA shape");
+  if (blockIdx.x < half) {
+    cellpipe(pass, gp, ps, blockIdx.x, half);
+    return;
+  }
+#pragma unroll 1
+  for (int l = src.cells1 ? 0 : 1; l < 2; ++l)
+    cellpass(pass, gp, src, l == 0 ? src.cells1 : src.cells, l == 0 ? src.ncells1 : src.ncells,
+             blockIdx.x - half, half);
+}
+
+template <class Pass>
+__global__ void __launch_bounds__(kPT, kPassBlocks) k_cells(Pass pass, const Grid* gp, PipeSrc ps,
+                                                            Src src, uint32_t half) {
+  dep_enter();
+  if (!pass.runs(*gp)) return;
+  run_pass(pass, gp, ps, src, half);
+}
+
+// The two forms as launches of their own.
+template <class Pass>
+__global__ void __launch_bounds__(kPT, kPassBlocks) k_cellpipe(Pass pass, const Grid* gp,
+                                                               PipeSrc ps) {
+  dep_enter();
+  if (!pass.runs(*gp)) return;
+  cellpipe(pass, gp, ps, blockIdx.x, gridDim.x);
+}
+template <class Pass>
+__global__ void __launch_bounds__(kPT, kPassBlocks) k_cellpass(Pass pass, const Grid* gp, Src src,
+                                                               const uint32_t* cells,
+                                                               const unsigned long long* ncells) {
+  dep_enter();
+  if (!pass.runs(*gp)) return;
+  cellpass(pass, gp, src, cells, ncells, blockIdx.x, gridDim.x);
+}
+
+template <class Pass>
+constexpr size_t pass_bytes() {
+  return PipeSmem<Pass>::kBytes > PassSmem<Pass>::kBytes ? PipeSmem<Pass>::kBytes
+                                                         : PassSmem<Pass>::kBytes;
+}
+
+// CTAs of one half of a pass launch.
+template <class K>
+int half_blocks(sph_ctx* ctx, K kernel, size_t smem, int* cache) {
   if (!*cache) {  // once per context, on its device
-    using SM = PipeSmem<Pass>;
-    cudaFuncSetAttribute(k_cellpipe<Pass>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)SM::kBytes);
-    cudaFuncSetAttribute(k_cellpipe<Pass>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                          (int)cudaSharedmemCarveoutMaxShared);
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cellpipe<Pass>, SM::PT,
-                                                  SM::kBytes);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kPT, smem);
     *cache = (per_sm > 0 ? per_sm : 1) * ctx->sm_count;
   }
   return *cache;
 }
 
-template <class Pass>
-int pass_blocks(sph_ctx* ctx, int* cache) {
-  if (!*cache) {  // once per context, on its device
-    using SM = PassSmem<Pass>;
-    cudaFuncSetAttribute(k_cellpass<Pass>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)SM::kBytes);
-    cudaFuncSetAttribute(k_cellpass<Pass>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         (int)cudaSharedmemCarveoutMaxShared);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cellpass<Pass>, kPT, SM::kBytes);
-    *cache = (per_sm > 0 ? per_sm : 1) * ctx->sm_count;
-  }
-  return *cache;
-}
-
-template <class Pass>
-void launch_pass(sph_ctx* ctx, const Pass& p, int* cache, cudaStream_t st) {
-  // the pipelined kernel: cells of at most 448 staged candidates, and for the
-  // passes with 16-byte records also those of 449..832
-  PipeSrc ps;
+// Cells of a pass: the pipelined form takes those of at most 448 staged
+// candidates, and for the passes with 16-byte records also those of 449..832.
+inline void pass_sources(sph_ctx* ctx, bool pipe_all, PipeSrc& ps, Src& src) {
   ps.meta = ctx->cmeta;
   ps.cells0 = ctx->cells;
   ps.n0 = ctx->salloc + 2;
-  ps.cells1 = Pass::kPipeAll ? ctx->cells + 2 * ctx->n_max : nullptr;
+  ps.cells1 = pipe_all ? ctx->cells + 2 * ctx->n_max : nullptr;
   ps.n1 = ctx->salloc + 4;
   ps.sent = ctx->sent;
   ps.nn = ctx->nn;
   ps.slist = reinterpret_cast<uint16_t*>(ctx->nbr);
   ps.max_nb = ctx->prm.max_nb;
-  launch_dep(k_cellpipe<Pass>, pipe_blocks<Pass>(ctx, cache + 3), Pass::kPipeThreads,
-      PipeSmem<Pass>::kBytes, st, p, ctx->grid, ps);
-  // the general kernel: the other cells (for momentum also those of 449..832)
-  Src src;
   src.meta = ctx->cmeta;
   src.sent = ctx->sent;
   src.nn = ctx->nn;
   src.nbr = ctx->nbr;
-  src.slist = reinterpret_cast<uint16_t*>(ctx->nbr);
+  src.slist = ps.slist;
   src.max_nb = ctx->prm.max_nb;
   src.cells = ctx->cells + ctx->n_max;
   src.ncells = ctx->salloc + 3;
-  launch_dep(k_cellpass<Pass>, pass_blocks<Pass>(ctx, cache), kPT, PassSmem<Pass>::kBytes, st, p,
-      ctx->grid, src);
-  ctx->launches += 2;
-  if (!Pass::kPipeAll) {
-    src.cells = ctx->cells + 2 * ctx->n_max;
-    src.ncells = ctx->salloc + 4;
-    launch_dep(k_cellpass<Pass>, pass_blocks<Pass>(ctx, cache), kPT, PassSmem<Pass>::kBytes, st,
-        p, ctx->grid, src);
-    ctx->launches += 1;
+  src.cells1 = pipe_all ? nullptr : ctx->cells + 2 * ctx->n_max;
+  src.ncells1 = ctx->salloc + 4;
+}
+
+// Momentum's common kernel takes 76 registers where the two forms alone take 70
+// and 74, and 2% longer at 8.4M particles (4.52 against 4.44 ms); side by side
+// saves 9 us of an 8,000-particle step.  From kSplitN particles on momentum
+// takes the forms alone.
+constexpr int64_t kSplitN = 1000000;
+
+template <class Pass>
+void launch_pass(sph_ctx* ctx, const Pass& p, int64_t n, int* cache, cudaStream_t st) {
+  PipeSrc ps;
+  Src src;
+  pass_sources(ctx, Pass::kPipeAll, ps, src);
+  constexpr size_t smem = pass_bytes<Pass>();
+  if constexpr (!Pass::kPipeAll) {
+    if (n >= kSplitN) {
+      constexpr size_t pipe = PipeSmem<Pass>::kBytes, pass = PassSmem<Pass>::kBytes;
+      launch_dep(k_cellpipe<Pass>, half_blocks(ctx, k_cellpipe<Pass>, pipe, cache + 1), kPT, pipe,
+                 st, p, ctx->grid, ps);
+      const int nb = half_blocks(ctx, k_cellpass<Pass>, pass, cache + 2);
+      launch_dep(k_cellpass<Pass>, nb, kPT, pass, st, p, ctx->grid, src, src.cells1, src.ncells1);
+      launch_dep(k_cellpass<Pass>, nb, kPT, pass, st, p, ctx->grid, src, src.cells, src.ncells);
+      ctx->launches += 3;
+      return;
+    }
   }
+  const int half = half_blocks(ctx, k_cells<Pass>, smem, cache);
+  launch_dep(k_cells<Pass>, 2 * half, kPT, smem, st, p, ctx->grid, ps, src, (uint32_t)half);
+  ctx->launches += 1;
 }
 
 // ----------------------------------------------------------------- export --
@@ -1728,13 +1835,16 @@ inline OutView outs_with_omega(const OutView& o, int gradh) {
 }  // namespace
 
 void launch_find_masks(sph_ctx* ctx, const StateView& s, int64_t n, cudaStream_t st) {
-  (void)n;
   const size_t smem = kFindWarps * (sizeof(FindWarpSmem) + kMaskBufWords * sizeof(unsigned long long));
   if (!ctx->find_mask_blocks) {  // once per context, on its device
     int per_sm = 0;
     cudaFuncSetAttribute(k_find_mask<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
     cudaFuncSetAttribute(k_find_mask<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+    cudaFuncSetAttribute(k_find_mask_cta<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+    cudaFuncSetAttribute(k_find_mask_cta<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_find_mask<false>, kFindThreads,
                                                   smem);
@@ -1752,12 +1862,23 @@ void launch_find_masks(sph_ctx* ctx, const StateView& s, int64_t n, cudaStream_t
   mo.scells = ctx->cells + ctx->n_max;
   mo.mcells = ctx->cells + 2 * ctx->n_max;
   cudaMemsetAsync(ctx->salloc, 0, 5 * sizeof(unsigned long long), st);
-  launch_dep(k_find_mask<false>, ctx->find_mask_blocks, kFindThreads, smem, st, ctx->grid, s,
-      ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb,
-      mo, ctx->err, ctx->stats);
-  launch_dep(k_find_mask<true>, ctx->find_mask_blocks, kFindThreads, smem, st, ctx->grid, s,
-      ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb,
-      mo, ctx->err, ctx->stats);
+  // One CTA per cell while the cells (of some 27 to 64 particles) hardly outnumber
+  // the SMs: a warp's search of a cell takes 55 us, most of it fetching and
+  // running code nobody shares (us, warp / CTA per cell: 4,096 particles 57 /
+  // 43, 8,000: 57 / 42, 13,824: 36 / 38, 21,952: 57 / 65).
+  const int64_t cta_max = 64 * (int64_t)ctx->sm_count;
+  auto run = [&](auto kernel) {
+    launch_dep(kernel, ctx->find_mask_blocks, kFindThreads, smem, st, ctx->grid, s, ctx->pos32,
+               ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb, mo,
+               ctx->err, ctx->stats);
+  };
+  if (n <= cta_max) {
+    run(k_find_mask_cta<false>);
+    run(k_find_mask_cta<true>);
+  } else {
+    run(k_find_mask<false>);
+    run(k_find_mask<true>);
+  }
   ctx->launches += 2;
 }
 
@@ -1772,22 +1893,23 @@ inline bool plain_kernel(const sph_ctx* ctx) {
 }
 
 template <template <int> class PassT, class Fill>
-void launch_cfg(sph_ctx* ctx, bool plain, int slot, Fill fill, cudaStream_t st) {
-  if (plain) {
-    PassT<kCfgPlain> q;
-    fill(q);
-    q.only_wrap = 0;
-    launch_pass(ctx, q, &ctx->pass_blocks[6 + slot], st);
-  }
-  PassT<kCfgAny> p;
+void launch_cfg(sph_ctx* ctx, bool plain, int slot, int64_t n, Fill fill, cudaStream_t st) {
+  using Plain = PassT<kCfgPlain>;
+  using Any = PassT<kCfgAny>;
+  Any p;
   fill(p);
   p.only_wrap = plain ? 1 : 0;
-  launch_pass(ctx, p, &ctx->pass_blocks[slot], st);
+  if (plain) {
+    Plain q;
+    fill(q);
+    q.only_wrap = 0;
+    launch_pass(ctx, q, n, ctx->pass_blocks[1][slot], st);
+  }
+  launch_pass(ctx, p, n, ctx->pass_blocks[0][slot], st);
 }
 
 void launch_density_staged(sph_ctx* ctx, const StateView& s, const OutView& o, int64_t n,
                            cudaStream_t st) {
-  (void)n;
   auto fill = [&](auto& p) {
     p.rec_d = ctx->rec_d;
     p.pos32 = ctx->pos32;
@@ -1803,13 +1925,12 @@ void launch_density_staged(sph_ctx* ctx, const StateView& s, const OutView& o, i
     p.gradh = ctx->prm.gradh;
     p.err = ctx->err;
   };
-  launch_cfg<DensityPassT>(ctx, plain_kernel(ctx) && !ctx->prm.gradh, 0, fill, st);
+  launch_cfg<DensityPassT>(ctx, plain_kernel(ctx) && !ctx->prm.gradh, 0, n, fill, st);
 }
 
 void launch_iad_staged(sph_ctx* ctx, const StateView& s, const OutView& o, int64_t n,
                        cudaStream_t st) {
   (void)s;
-  (void)n;
   auto fill = [&](auto& p) {
     p.rec_i = ctx->rec_i;
     p.recA = ctx->recA;
@@ -1822,13 +1943,12 @@ void launch_iad_staged(sph_ctx* ctx, const StateView& s, const OutView& o, int64
     p.sinc_n = (int)ctx->prm.sinc_n;
     p.err = ctx->err;
   };
-  launch_cfg<IadPassT>(ctx, plain_kernel(ctx) && !ctx->prm.gradh, 1, fill, st);
+  launch_cfg<IadPassT>(ctx, plain_kernel(ctx) && !ctx->prm.gradh, 1, n, fill, st);
 }
 
 void launch_momentum_staged(sph_ctx* ctx, const StateView& s, const OutView& o, int64_t n,
                             cudaStream_t st) {
   (void)s;
-  (void)n;
   auto fill = [&](auto& p) {
     p.recA = ctx->recA;
     p.recV = ctx->recV;
@@ -1843,7 +1963,7 @@ void launch_momentum_staged(sph_ctx* ctx, const StateView& s, const OutView& o, 
     p.inv_gamma = (float)(1.0 / ctx->prm.gamma);
     p.err = ctx->err;
   };
-  launch_cfg<MomentumPassT>(ctx, plain_kernel(ctx) && !ctx->prm.gradh, 2, fill, st);
+  launch_cfg<MomentumPassT>(ctx, plain_kernel(ctx) && !ctx->prm.gradh, 2, n, fill, st);
 }
 
 void launch_export_masks(sph_ctx* ctx, const StateView& s, int64_t n, int32_t* counts,

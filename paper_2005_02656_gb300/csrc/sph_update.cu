@@ -27,7 +27,9 @@ namespace sph {
 
 namespace {
 
-constexpr int kThreads = 256;
+// 128-thread blocks: a small state then spreads over more SMs, and the FP64 pipe
+// (one warp instruction per 64 cycles and quarter SM) bounds these kernels.
+constexpr int kThreads = 128;
 constexpr int kParts = 16;  // doubles per block partial
 
 __device__ __forceinline__ bool block_last(unsigned int* counter) {
@@ -42,16 +44,39 @@ __device__ __forceinline__ bool block_last(unsigned int* counter) {
   return last;
 }
 
-// Block sum of NV doubles per thread into part[blockIdx.x * kParts + k].
-template <int NV>
-__device__ __forceinline__ void block_sums(double (&v)[NV], double* part) {
-  __shared__ double sh[kThreads / 32][NV];
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
+// Sums of 8 doubles over the warp: a transposing butterfly (9 additions a lane
+// instead of 40).  Lane l < 8 returns the sum of v[slot8(l)].
+__device__ __forceinline__ int slot8(int lane) {
+  return ((lane & 1) << 2) | (lane & 2) | ((lane >> 2) & 1);
+}
+__device__ __forceinline__ double warp_sums8(const double (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+  double r[4], q[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const bool up = lane & 1;
+    r[i] = (up ? v[4 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[4 + i], 1);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const bool up = lane & 2;
+    q[i] = (up ? r[2 + i] : r[i]) + __shfl_xor_sync(0xffffffffu, up ? r[i] : r[2 + i], 2);
+  }
+  const bool up = lane & 4;
+  double t = (up ? q[1] : q[0]) + __shfl_xor_sync(0xffffffffu, up ? q[0] : q[1], 4);
+  t += __shfl_xor_sync(0xffffffffu, t, 8);
+  t += __shfl_xor_sync(0xffffffffu, t, 16);
+  return t;
+}
+
+// Block sums of 8 doubles per thread into part[blockIdx.x * kParts + k].
+__device__ __forceinline__ void block_sums8(const double (&v)[8], double* part) {
+  __shared__ double sh[kThreads / 32][8];
+  const double t = warp_sums8(v);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0)
-    for (int k = 0; k < NV; ++k) sh[w][k] = v[k];
+  if (l < 8) sh[w][slot8(l)] = t;
   __syncthreads();
-  if (threadIdx.x < NV) {
+  if (threadIdx.x < 8) {
     double s = 0.0;
     for (int ww = 0; ww < kThreads / 32; ++ww) s += sh[ww][threadIdx.x];
     part[blockIdx.x * kParts + threadIdx.x] = s;
@@ -59,11 +84,11 @@ __device__ __forceinline__ void block_sums(double (&v)[NV], double* part) {
 }
 
 // The last block's reduction of the per-block partials part[b * kParts + k]:
-// every thread takes the blocks b = tid, tid + blockDim, ... in order, then a
-// fixed-shape warp and block tree combines them, so the result does not
-// depend on timing.  Reads go to L2 (the partials were written by other
-// blocks before their fence and counter increment).  Called by all threads of
-// the block; out (shared) receives the NV results.
+// warp w takes the values k = w, w + 4, ..., its lanes the blocks b = lane,
+// lane + 32, ... in order, then a fixed-shape butterfly combines them, so the
+// result does not depend on timing.  Reads go to L2 (the partials were written
+// by other blocks before their fence and counter increment).  Called by all
+// threads of the block; out (shared) receives the NV results.
 enum class Op { kSum, kMin, kMax };
 
 __device__ __forceinline__ double op_apply(Op op, double a, double b) {
@@ -73,27 +98,15 @@ __device__ __forceinline__ double op_apply(Op op, double a, double b) {
 template <int NV>
 __device__ void finalize_block(const double* part, int nblocks, const Op (&op)[NV],
                                double* out) {
-  __shared__ double sh[kThreads / 32][NV];
-  double v[NV];
-#pragma unroll
-  for (int k = 0; k < NV; ++k)
-    v[k] = op[k] == Op::kSum ? 0.0 : (op[k] == Op::kMin ? INFINITY : -INFINITY);
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = op_apply(op[k], v[k], __ldcg(part + b * kParts + k));
-#pragma unroll
-  for (int k = 0; k < NV; ++k)
-    for (int o = 16; o > 0; o >>= 1) v[k] = op_apply(op[k], v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0)
 #pragma unroll
-    for (int k = 0; k < NV; ++k) sh[w][k] = v[k];
-  __syncthreads();
-  if (threadIdx.x < NV) {
-    const int k = threadIdx.x;
-    double r = sh[0][k];
-    for (int ww = 1; ww < (int)(blockDim.x >> 5); ++ww) r = op_apply(op[k], r, sh[ww][k]);
-    out[k] = r;
+  for (int k = 0; k < NV; ++k) {
+    if (k % (kThreads / 32) != w) continue;
+    double v = op[k] == Op::kSum ? 0.0 : (op[k] == Op::kMin ? INFINITY : -INFINITY);
+    for (int b = l; b < nblocks; b += 32) v = op_apply(op[k], v, __ldcg(part + b * kParts + k));
+    for (int o = 16; o > 0; o >>= 1)
+      v = op_apply(op[k], v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (l == 0) out[k] = v;
   }
   __syncthreads();
 }
@@ -114,6 +127,14 @@ __device__ __forceinline__ float f32_of_hi(double v) {
 // quotient whose q32 exceeds the running minimum's FP32 value by the factor
 // 1 + 2^-16 is larger than that minimum and needs no FP64 division.
 constexpr float kScreen = 1.0f + 0x1p-16f;
+
+// Warp minimum on ordered integer keys (fmin would take a NaN for the larger
+// value; running minima hold none).
+__device__ __forceinline__ double warp_min_key(double v) {
+  long long k = okey(v, kKeyInf);
+  for (int o = 16; o > 0; o >>= 1) k = min(k, __shfl_xor_sync(0xffffffffu, k, o));
+  return from_okey(k);
+}
 
 __global__ void __launch_bounds__(kThreads) k_timestep(const double* h, const double* c,
                                                        const double* u, const double* du,
@@ -150,8 +171,8 @@ __global__ void __launch_bounds__(kThreads) k_timestep(const double* h, const do
       }
     }
   }
-  mn = warp_min(mn);
-  mu = warp_min(mu);
+  mn = warp_min_key(mn);
+  if (energy_dt > 0.0) mu = warp_min_key(mu);
   __shared__ double sh[2][kThreads / 32];
   if ((threadIdx.x & 31) == 0) {
     sh[0][threadIdx.x >> 5] = mn;
@@ -211,7 +232,7 @@ __global__ void __launch_bounds__(kThreads) k_update(StateView s, OutView o, Sta
   const double dt = diag[8], dt_prev = diag[12];
   const double delta = 0.5 * (dt + dt_prev);
   const double q = dt_prev > 0.0 ? dt / (2.0 * dt_prev) : 0.0;
-  double acc[11] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   // periodic wrap tests on ordered integer keys of the box corners (a NaN
   // position takes the key of box_lo: no wrap, as in the FP comparison)
   long long klo[3], khi[3];
@@ -221,8 +242,8 @@ __global__ void __launch_bounds__(kThreads) k_update(StateView s, OutView o, Sta
     khi[k] = okey(prm.box_hi[k], 0);
   }
   // neighbour-count statistics in integer arithmetic (FP64 runs at 1/64 of the
-  // FP32 rate on this part); converted once per thread below
-  long long csum = 0;
+  // FP32 rate on this part); converted once per block below
+  uint32_t csum = 0;  // per thread at most 2^27 / 155,648 counts of 65,535: a warp's sum fits 32 bits
   int cmin = INT_MAX, cmax = INT_MIN;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
        p += (int64_t)gridDim.x * blockDim.x) {
@@ -282,31 +303,30 @@ __global__ void __launch_bounds__(kThreads) k_update(StateView s, OutView o, Sta
       acc[6] += m * (xn[2] * vn[0] - xn[0] * vn[2]);
       acc[7] += m * (xn[0] * vn[1] - xn[1] * vn[0]);
     }
-    csum += cnt;
+    csum += (uint32_t)cnt;
     cmin = min(cmin, cnt);
     cmax = max(cmax, cnt);
   }
-  acc[8] = 0.0;
-  acc[9] = 0.0;
-  acc[10] = (double)csum;  // exact: the sum is far below 2^53
-  double nmin = cmin == INT_MAX ? INFINITY : (double)cmin;
-  double nmax = cmax == INT_MIN ? -INFINITY : (double)cmax;
-  nmin = warp_min(nmin);
-  nmax = warp_max(nmax);
-  __shared__ double shm[kThreads / 32][2];
+  csum = __reduce_add_sync(0xffffffffu, csum);
+  cmin = __reduce_min_sync(0xffffffffu, cmin);
+  cmax = __reduce_max_sync(0xffffffffu, cmax);
+  __shared__ int shm[kThreads / 32][3];
   if ((threadIdx.x & 31) == 0) {
-    shm[threadIdx.x >> 5][0] = nmin;
-    shm[threadIdx.x >> 5][1] = nmax;
+    shm[threadIdx.x >> 5][0] = (int)csum;
+    shm[threadIdx.x >> 5][1] = cmin;
+    shm[threadIdx.x >> 5][2] = cmax;
   }
-  block_sums<11>(acc, part);
-  __syncthreads();
+  block_sums8(acc, part);
   if (threadIdx.x == 0) {
+    unsigned long long total = csum;
     for (int w = 1; w < kThreads / 32; ++w) {
-      nmin = fmin(nmin, shm[w][0]);
-      nmax = fmax(nmax, shm[w][1]);
+      total += (uint32_t)shm[w][0];
+      cmin = min(cmin, shm[w][1]);
+      cmax = max(cmax, shm[w][2]);
     }
-    part[blockIdx.x * kParts + 8] = nmin;
-    part[blockIdx.x * kParts + 9] = nmax;
+    part[blockIdx.x * kParts + 8] = cmin == INT_MAX ? INFINITY : (double)cmin;
+    part[blockIdx.x * kParts + 9] = cmax == INT_MIN ? -INFINITY : (double)cmax;
+    part[blockIdx.x * kParts + 10] = (double)total;  // exact: the sum is far below 2^53
   }
   if (!block_last(counter)) return;
   __threadfence();
@@ -343,7 +363,7 @@ __global__ void __launch_bounds__(kThreads) k_diag(StateView s, int64_t n, doubl
     acc[6] += m * (z * vx - x * vz);
     acc[7] += m * (x * vy - y * vx);
   }
-  block_sums<8>(acc, part);
+  block_sums8(acc, part);
   if (!block_last(counter)) return;
   __threadfence();
   __shared__ double res[8];
@@ -356,7 +376,7 @@ __global__ void __launch_bounds__(kThreads) k_diag(StateView s, int64_t n, doubl
 
 inline int red_blocks(int64_t n, int sm) {
   int64_t b = (n + kThreads - 1) / kThreads;
-  int64_t cap = (int64_t)sm * 4;
+  int64_t cap = (int64_t)sm * 8;
   if (cap > kReduceBlocks) cap = kReduceBlocks;
   if (b > cap) b = cap;
   if (b < 1) b = 1;
