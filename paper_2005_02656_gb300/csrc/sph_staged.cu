@@ -1861,7 +1861,6 @@ void launch_find_masks(sph_ctx* ctx, const StateView& s, int64_t n, cudaStream_t
   mo.fcells = ctx->cells;
   mo.scells = ctx->cells + ctx->n_max;
   mo.mcells = ctx->cells + 2 * ctx->n_max;
-  cudaMemsetAsync(ctx->salloc, 0, 5 * sizeof(unsigned long long), st);
   // One CTA per cell while the cells (of some 27 to 64 particles) hardly outnumber
   // the SMs: a warp's search of a cell takes 55 us, most of it fetching and
   // running code nobody shares (us, warp / CTA per cell: 4,096 particles 57 /
