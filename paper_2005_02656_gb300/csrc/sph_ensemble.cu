@@ -460,7 +460,7 @@ __device__ void ph_gather(const Args& A) {
     const float m32 = f32_rn(m);
     A.pos32[p] = make_float4(ox, oy, oz, f32_rn(h));
     A.rec_d[p] = make_float4(ox, oy, oz, m32);
-    A.rec_m[5 * p + 1] = make_float4(f32_rn(vx), f32_rn(vy), f32_rn(vz), m32);
+    A.rec_m[A.n + p] = make_float4(f32_rn(vx), f32_rn(vy), f32_rn(vz), m32);
   }
 }
 
@@ -491,6 +491,7 @@ __device__ __forceinline__ pairs32::F32 f32_of(const Args& A) {
   f.rec_d = A.rec_d;
   f.rec_i = A.rec_i;
   f.rec_m = A.rec_m;
+  f.ms = (uint32_t)A.n;
   f.ktab = nullptr;  // the ensemble runs the exact kernel
   return f;
 }
@@ -1038,7 +1039,7 @@ int sph_ensemble_init(const sph_params* common, int n_boxes, const int64_t* box_
   A((void**)&e->pos32, 16 * N);
   A((void**)&e->rec_d, 16 * N);
   A((void**)&e->rec_i, 16 * N);
-  A((void**)&e->rec_m, 80 * N);
+  A((void**)&e->rec_m, 72 * N);
   A((void**)&e->nn, 4 * N);
   A((void**)&e->nbr, 4 * N * (size_t)common->max_nb);
   A((void**)&e->hfac, 8 * (size_t)(sph::kMaxSlots + 1));

@@ -122,7 +122,7 @@ struct sph_ctx {
   // FP32 mixed-path per-particle records (sorted order, sph_pairs_fp32.cu)
   float4* rec_d;        // offset x, y, z, m               (gather)
   float4* rec_i;        // offset x, y, z, m/rho           (density)
-  float4* rec_m;        // 5 float4 per particle           (gather, density, IAD)
+  float4* rec_m;        // 4 float4 planes, a float2 plane (gather, density, IAD)
 
   // SPH_PAIRS_STAGED (sph_staged.cu): per occupied cell (slot_base,
   // mask_base, a0, S << 16 | na); staged candidate entries; hit masks

@@ -10,8 +10,11 @@
 // gathered through L1/L2 from packed records:
 //   rec_d (density)  = (offset x, y, z, m)                       16 B
 //   rec_i (IAD)      = (offset x, y, z, m/rho)                   16 B
-//   rec_m (momentum) = (offset, 1/h^2), (v, m), (B_n/h^3, P/rho^2, c, 1/rho),
-//                      (C00 C01 C02 C11), (C12 C22 - -)          80 B
+//   rec_m (momentum) = planes (offset, 1/h^2), (v, m), (B_n/h^3, P/rho^2, c, 1/rho),
+//                      (C00 C01 C02 C11), (C12 C22)              72 B
+// The four lanes that share a momentum target take consecutive entries of its
+// list, which lie a few particles apart: a plane's four values share one or two
+// 128-byte lines, where 80-byte records put each on a line of its own.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -27,7 +30,14 @@ struct F32 {
   const float4* pos;    // offset in own cell x, y, z, h
   const float4* rec_d;  // offset x, y, z, m
   float4* rec_i;        // offset x, y, z, m/rho
-  float4* rec_m;        // 5 float4 per particle
+  float4* rec_m;        // four float4 planes and one float2 plane of ms particles
+  uint32_t ms;
+
+  // 32-bit indices (5 x 2^27 at most) keep one base pointer in registers, not five
+  __device__ __forceinline__ float4& m(uint32_t q, uint32_t i) const { return rec_m[q * ms + i]; }
+  __device__ __forceinline__ float2& m4(uint32_t i) const {
+    return reinterpret_cast<float2*>(rec_m)[8u * ms + i];
+  }
   const float2* ktab;   // SPH_KERNEL_TABLE values, NULL for the exact kernel
 };
 
@@ -168,15 +178,14 @@ __device__ __forceinline__ void density_one(int64_t a, const Grid& g, const F32&
   o.c[a] = c;
   const float inv_rho = 1.0f / rho;
   f.rec_i[a] = make_float4(pa.x, pa.y, pa.z, ma * inv_rho);
-  float4* m = f.rec_m + 5 * a;
-  m[0] = make_float4(pa.x, pa.y, pa.z, hinv2);
+  f.m(0, (uint32_t)a) = make_float4(pa.x, pa.y, pa.z, hinv2);
   double X = p / (rho64 * rho64);
   if (gradh) {
     const double omega = -2.0 * (double)gsum / (3.0 * rho64);
     X /= omega;
     if (o.omega) o.omega[a] = omega;
   }
-  m[2] = make_float4(norm, (float)X, (float)c, inv_rho);
+  f.m(2, (uint32_t)a) = make_float4(norm, (float)X, (float)c, inv_rho);
   if (!isfinite(rho64) || !isfinite(c)) raise_flag(err, SPH_FLAG_NONFINITE);
 }
 
@@ -193,8 +202,8 @@ __device__ __forceinline__ void iad_one(int64_t a, const Grid& g, const F32& f, 
   float hinv2 = 0.f;
   if (on) {
     const float4 pa = f.pos[a];
-    hinv2 = f.rec_m[5 * a].w;
-    const float norm = f.rec_m[5 * a + 2].x;
+    hinv2 = f.m(0, (uint32_t)a).w;
+    const float norm = f.m(2, (uint32_t)a).x;
     const int cnt = min(L.nn[a], L.max_nb);
     for_entries_part<NSUB>(L.nbr + a * L.max_nb, cnt, sub, [&](uint32_t e) {
       const float4 rb = f.rec_i[entry_index(e)];
@@ -241,9 +250,8 @@ __device__ __forceinline__ void iad_one(int64_t a, const Grid& g, const F32& f, 
     Cm[4] = c12 * sc;
     Cm[5] = c22 * sc;
   }
-  float4* m = f.rec_m + 5 * a;
-  m[3] = make_float4(Cm[0], Cm[1], Cm[2], Cm[3]);
-  m[4] = make_float4(Cm[4], Cm[5], 0.0f, 0.0f);
+  f.m(3, (uint32_t)a) = make_float4(Cm[0], Cm[1], Cm[2], Cm[3]);
+  f.m4((uint32_t)a) = make_float2(Cm[4], Cm[5]);
   double* out = o.iad + 6 * a;
   for (int q = 0; q < 6; ++q) out[q] = (double)Cm[q];
 }
@@ -259,22 +267,22 @@ __device__ __forceinline__ void momentum_one(int64_t a, const Grid& g, const F32
   if (N > 0) sinc_n = N;
   float accx = 0, accy = 0, accz = 0, du = 0;
   if (on) {
-    const float4* ra = f.rec_m + 5 * a;
-    const float4 pa = ra[0];       // offset, 1/h_a^2
-    const float4 va = ra[1];       // v, m
-    const float4 qa = ra[2];       // B_n/h^3, P/rho^2, c, 1/rho
-    const float4 Aa = ra[3], Ba = ra[4];
+    const float4 pa = f.m(0, (uint32_t)a);   // offset, 1/h_a^2
+    const float4 va = f.m(1, (uint32_t)a);   // v, m
+    const float4 qa = f.m(2, (uint32_t)a);   // B_n/h^3, P/rho^2, c, 1/rho
+    const float4 Aa = f.m(3, (uint32_t)a);
+    const float2 Ba = f.m4((uint32_t)a);
     const float a00 = Aa.x, a01 = Aa.y, a02 = Aa.z, a11 = Aa.w, a12 = Ba.x, a22 = Ba.y;
     const float Xa = qa.y, csa = qa.z, ira = qa.w;
     const int cnt = min(L.nn[a], L.max_nb);
     for_entries_part<NSUB>(L.nbr + a * L.max_nb, cnt, sub, [&](uint32_t e) {
       // one pair of Eqs. 2-5 (x_ab = -d, d = x_b - x_a)
-      const float4* rb = f.rec_m + 5 * (int64_t)entry_index(e);
-      const float4 b0 = rb[0];
+      const uint32_t b = (uint32_t)entry_index(e);
+      const float4 b0 = f.m(0, b);
       float dx, dy, dz;
       rel(g, wrap, e, b0, pa, dx, dy, dz);
       const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-      const float4 b2 = rb[2];
+      const float4 b2 = f.m(2, b);
       // W_a and W_b together in paired FP32, clamped at t = 4 (S = 0)
       const float2 Wab = kw32x2(make_float2(r2 * pa.w, r2 * b0.w), make_float2(qa.x, b2.x),
                                 sinc_n, f.ktab);
@@ -282,11 +290,12 @@ __device__ __forceinline__ void momentum_one(int64_t a, const Grid& g, const F32
       const float Cadx = fmaf(a02, dz, fmaf(a01, dy, a00 * dx));
       const float Cady = fmaf(a12, dz, fmaf(a11, dy, a01 * dx));
       const float Cadz = fmaf(a22, dz, fmaf(a12, dy, a02 * dx));
-      const float4 b3 = rb[3], b4 = rb[4];
+      const float4 b3 = f.m(3, b);
+      const float2 b4 = f.m4(b);
       const float Cbdx = fmaf(b3.z, dz, fmaf(b3.y, dy, b3.x * dx));
       const float Cbdy = fmaf(b4.x, dz, fmaf(b3.w, dy, b3.y * dx));
       const float Cbdz = fmaf(b4.y, dz, fmaf(b4.x, dy, b3.z * dx));
-      const float4 vb = rb[1];
+      const float4 vb = f.m(1, b);
       const float vabx = va.x - vb.x, vaby = va.y - vb.y, vabz = va.z - vb.z;
       const float xv = -fmaf(dz, vabz, fmaf(dy, vaby, dx * vabx));
       // Eq. 5 without a branch: w_ab = x_ab.v_ab / r, Pi = 0 unless approaching

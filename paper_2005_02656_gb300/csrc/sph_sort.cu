@@ -433,7 +433,7 @@ __global__ void k_gather_a(StateView in, StateView out, int64_t n, const double*
 // the momentum pass (so a caller may still be copying them in while the
 // search runs).  Loads before stores, as in k_gather_a.
 __global__ void k_gather_b(StateView in, StateView out, int64_t n, const int32_t* perm,
-                           float4* rec_m, float4* recV) {
+                           float4* vplane) {
   dep_enter();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -451,11 +451,7 @@ __global__ void k_gather_b(StateView in, StateView out, int64_t n, const int32_t
     out.vyh[p] = vyh;
     out.vzh[p] = vzh;
     out.du_prev[p] = dup;
-    const float4 vm = make_float4(f32_rn(vx), f32_rn(vy), f32_rn(vz), f32_rn(m));
-    if (recV)
-      recV[p] = vm;  // the staged pair passes' velocity plane
-    else
-      rec_m[5 * p + 1] = vm;
+    vplane[p] = make_float4(f32_rn(vx), f32_rn(vy), f32_rn(vz), f32_rn(m));
     s = s_next;
   }
 }
@@ -529,7 +525,7 @@ void launch_sort(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st,
 
 void launch_gather_b(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st) {
   launch_dep(k_gather_b, grid_for(n, 256, ctx->sm_count), 256, 0, st, in, ctx->s, n, ctx->perm,
-      ctx->rec_m, staged_pairs(ctx) ? ctx->recV : nullptr);
+      staged_pairs(ctx) ? ctx->recV : ctx->rec_m + ctx->n_max);
   ctx->launches += 1;
 }
 
