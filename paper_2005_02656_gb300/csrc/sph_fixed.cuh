@@ -17,12 +17,18 @@ namespace fx {
 
 #ifdef __CUDA_ARCH__
 #define SPH_FX __device__ __forceinline__
+SPH_FX float rsqrt32(float a) { return rsqrtf(a); }
+SPH_FX uint32_t bits_of(float v) { return __float_as_uint(v); }
+SPH_FX float from_bits(uint32_t b) { return __uint_as_float(b); }
 SPH_FX uint32_t mulhi32(uint32_t a, uint32_t b) { return __umulhi(a, b); }
 SPH_FX int clz64(uint64_t a) { return __clzll((long long)a); }
 SPH_FX uint64_t bits_of(double v) { return (uint64_t)__double_as_longlong(v); }
 SPH_FX double from_bits(uint64_t b) { return __longlong_as_double((long long)b); }
 #else
 #define SPH_FX inline
+SPH_FX float rsqrt32(float a) { return (float)(1.0 / __builtin_sqrt((double)a)); }
+SPH_FX uint32_t bits_of(float v) { uint32_t b; __builtin_memcpy(&b, &v, 4); return b; }
+SPH_FX float from_bits(uint32_t b) { float v; __builtin_memcpy(&v, &b, 4); return v; }
 SPH_FX uint32_t mulhi32(uint32_t a, uint32_t b) { return (uint32_t)(((uint64_t)a * b) >> 32); }
 SPH_FX int clz64(uint64_t a) { return a ? __builtin_clzll(a) : 64; }
 SPH_FX uint64_t bits_of(double v) { uint64_t b; __builtin_memcpy(&b, &v, 8); return b; }
@@ -124,6 +130,28 @@ SPH_FX double S6(double t) {
   return pack(mulhi64(mulhi64(m2, m2), m2), 6 - 6 * z);
 }
 
+// S^6 at the fraction y, and a S^6: the mantissas are multiplied before the one
+// rounding to a double (a normal and not near the ends of the range, or the
+// product is taken in FP64).
+SPH_FX double S6_at(uint64_t y) {
+  const uint64_t s = sinc(y);
+  if (s == 0) return 0.0;
+  const int z = clz64(s);
+  const uint64_t m = s << z, m2 = mulhi64(m, m);
+  return pack(mulhi64(mulhi64(m2, m2), m2), 6 - 6 * z);
+}
+SPH_FX double S6_at_times(uint64_t y, double a) {
+  const uint64_t b = bits_of(a);
+  const int E = (int)(b >> 52) & 0x7ff;
+  if (E < 512 || E > 1535) return a * S6_at(y);
+  const uint64_t s = sinc(y);
+  if (s == 0) return 0.0;
+  const int z = clz64(s);
+  const uint64_t m = s << z, m2 = mulhi64(m, m);
+  const uint64_t f = mulhi64(mulhi64(mulhi64(m2, m2), m2), (b << 11) | 0x8000000000000000u);
+  return from_bits(bits_of(pack(f, 6 - 6 * z + E - 1022)) | (b & 0x8000000000000000u));
+}
+
 // S^6 and its derivative by t, 6 S^5 dS/dt (dS/dt = (dS/dy) / 4).
 SPH_FX void S6_d(double t, double& w, double& dw) {
   w = dw = 0.0;
@@ -157,7 +185,8 @@ SPH_FX int64_t fixed(double v, int eb) {
   const uint64_t b = bits_of(v);
   const int s = eb - (int)((b >> 52) & 0x7ffu);  // >= 1
   uint64_t m = (b & 0xfffffffffffffu) << (N - 52) | (uint64_t)1 << N;
-  m >>= (unsigned)s < 63u ? s : 63;  // |v| beyond the power of two: no value, but no overflow
+  m >>= (unsigned)s < 63u ? s : 63;
+  if (s <= 0) m = ((uint64_t)1 << N) - 1;  // |v| not below the power of two: the largest value
   const int64_t g = (int64_t)b >> 63;
   return ((int64_t)m ^ g) - g;
 }
@@ -197,6 +226,75 @@ SPH_FX double scaled(int64_t x, int k) {
   const uint64_t m = u << z;
   return from_bits((((uint64_t)(uint32_t)f << 52) + (m >> 11) + ((m >> 10) & 1u)) |
                    ((uint64_t)g << 63));
+}
+
+// y = t / 4 = r^2 / (4 h^2) in units of 2^-64 from R = r^2 2^-k (R < 2^60) and
+// 1 / h^2 (normal); false where t >= 4.
+SPH_FX bool fraction_of(uint64_t R, int k, double hinv2, uint64_t& y) {
+  const uint64_t b = bits_of(hinv2);
+  // 1 / h^2 = H 2^(E - 1086), H in [2^63, 2^64)
+  const uint64_t p = mulhi64(R << 3, (b << 11) | 0x8000000000000000u);  // R H 2^-61
+  const int s = (int)(b >> 52) - 1086 + 61 + 62 + k;                    // y 2^64 = p 2^s
+  y = 0;
+  if (s <= 0) {
+    y = p >> (s > -63 ? -s : 63);
+    return true;
+  }
+  if (s > 63 ? p != 0 : (p >> (64 - s)) != 0) return false;
+  y = s > 63 ? 0 : p << s;
+  return true;
+}
+
+// A positive double of the middle of the range as m 2^(e - 64), m in [2^62, 2^64)
+// (products of two such values included).
+struct Mant {
+  uint64_t m;
+  int e;
+};
+SPH_FX bool middle(double a) {
+  const uint64_t b = bits_of(a);
+  return (b >> 52) - 823u < 400u;  // positive, 2^-200 <= a < 2^200
+}
+SPH_FX Mant mant(double a) {
+  const uint64_t b = bits_of(a);
+  return {(b << 11) | 0x8000000000000000u, (int)(b >> 52) - 1022};
+}
+SPH_FX Mant operator*(const Mant& a, const Mant& b) { return {mulhi64(a.m, b.m), a.e + b.e}; }
+
+// a x for x in fixed point (units 2^k, |x| < 2^61).
+SPH_FX double times(const Mant& a, int64_t x, int k) {
+  const int64_t g = x >> 63;
+  const uint64_t u = (uint64_t)((x ^ g) - g);
+  const uint64_t f = mulhi64(a.m, u << 3);  // a x 2^-k 2^(3 - e)
+  if (f == 0) return 0.0;
+  return from_bits(bits_of(pack(f, a.e + k + 61)) | ((uint64_t)g << 63));
+}
+
+// v 2^kv / sqrt(R 2^kr) for v != 0 and R >= 2^52 (whose error of a unit is then
+// below 2^-52): y0 from the FP32 reciprocal square root, and the factor
+// 1 + e/2 + 3 e^2/8 with e = 1 - R y0^2, in 64-bit fixed point.
+SPH_FX double over_root(int64_t v, int kv, uint64_t R, int kr) {
+  int z = clz64(R);
+  uint64_t m = R << z;  // m 2^-62 in [2, 4)
+  int x = 62 - z + kr;
+  if (x & 1) {
+    m >>= 1;            // [1, 2)
+    ++x;
+  }
+  const float y0 = rsqrt32((float)(uint32_t)(m >> 32) * 9.313225746154785e-10f);  // 2^-30
+  const uint32_t Y = (uint32_t)(y0 * 2147483648.0f);                             // y0 2^31, exact
+  const int64_t e = (int64_t)0x2000000000000000 - (int64_t)mulhi64(m, ((uint64_t)Y * Y) << 1);
+  const int64_t e20 = e >> 20;
+  const int64_t q = (e >> 1) + ((3 * e20 * e20) >> 24);                          // 2^61
+  const int64_t g = v >> 63;
+  const uint64_t u = (uint64_t)((v ^ g) - g);
+  const int zv = clz64(u);
+  const uint64_t n = u << zv;
+  uint64_t t = (uint64_t)(uint32_t)(n >> 32) * Y + mulhi32((uint32_t)n, Y);      // n y0 / 2
+  t = q < 0 ? t - mulhi64(t, (uint64_t)-q << 3) : t + mulhi64(t, (uint64_t)q << 3);
+  const int ex = 65 - zv + kv - (x >> 1);  // result t 2^(ex - 64)
+  if (ex < -900 || ex > 900) return 0.0 * (double)g;
+  return from_bits(bits_of(pack(t, ex)) | ((uint64_t)g << 63));
 }
 
 }  // namespace fx

@@ -15,10 +15,12 @@
 //    only in warps that hold a pair across a boundary;
 //  - 1/r takes its seed from the FP32 reciprocal square root, and per-pair
 //    divisions are hoisted into per-particle arrays;
+//  - scalar products are block fixed point, and with S^6 (FAST) so are r^2, v
+//    and 1/r, from the separation's fixed-point form;
 //  - the per-target work runs on whole warps (lanes_sum).
-// Per pair 8 (density), 13 (IAD) and 37 (momentum) FP64 operations; at 1.07M
-// particles 2.64, 3.77 and 9.7 ms, where the FP64 series, FP comparisons and
-// one thread per target took 7.38, 4.11 and 20.6 ms.
+// Per pair about 4 (density), 9 (IAD) and 28 (momentum) FP64 operations; at
+// 1.07M particles 1.82, 2.86 and 7.99 ms, where the FP64 series, products and
+// comparisons with one thread per target took 7.38, 4.11 and 20.6 ms.
 #include <cuda_runtime.h>
 #include "sph_device.cuh"
 #include "sph_fixed.cuh"
@@ -56,12 +58,30 @@ __device__ __forceinline__ double shape64(double t, int n, const double2* tab) {
   return n == 6 ? fx::S6(t) : ipow(fx::S(t), n);
 }
 
+// A vector in block fixed point with the given power of two.
+__device__ __forceinline__ fx::Vec3 vec64(double x, double y, double z, int eb) {
+  fx::Vec3 v;
+  fx::put(v, 0, fx::fixed<61>(x, eb));
+  fx::put(v, 1, fx::fixed<61>(y, eb));
+  fx::put(v, 2, fx::fixed<61>(z, eb));
+  return v;
+}
+
+// S^6 of r^2 = R 2^k and 1 / h^2; 0 from the support's edge on (R reaches 2^60 at
+// the target's own).
+__device__ __forceinline__ double shape_at(int64_t R, int k, double hinv2) {
+  uint64_t y;
+  return (uint64_t)R >> 60 == 0 && fx::fraction_of((uint64_t)R, k, hinv2, y) ? fx::S6_at(y) : 0.0;
+}
+
 // GRADH: also the grad-h terms, Omega_a = 1 + h_a/(3 rho_a) sum_b m_b dW/dh_a.
 // With dW/dh = -(3 W + v dW/dv) / h and sum_b m_b W = rho_a (self term
 // included) this is Omega_a = -(2 / (3 rho_a)) sum_{b != a} m_b t dW/dt,
 // t = v^2 (the self term has t = 0); X = P / (Omega rho^2) then carries it
 // into Eqs. 2-3.
-template <int NSUB, bool GRADH>
+// FAST (the default kernel: exact, n = 6, no grad-h terms): t and S^6 in fixed
+// point from the components of d, so that 4 FP64 operations per pair are left.
+template <int NSUB, bool GRADH, bool FAST>
 __global__ void __launch_bounds__(kThreads64) k_density64(const Grid* gp, StateView s, OutView o,
                                                           Aux64 aux, Lists64 L, int64_t n,
                                                           double Bn, int sinc_n, double gamma,
@@ -85,13 +105,21 @@ __global__ void __launch_bounds__(kThreads64) k_density64(const Grid* gp, StateV
   double acc = 0.0, gsum = 0.0;
   __syncthreads();
   const double hinv2 = sh_hinv2[t_loc];
+  const int ed = fx::exp_above(2.0 * s.h[a]);  // |d| < 2 h_a
   for (int k = sub; k < cnt; k += NSUB) {
     const int64_t b = entry_index(list[k]);
     double dx = s.x[b] - xa, dy = s.y[b] - ya, dz = s.z[b] - za;
     sep64(im, dx, dy, dz);
-    const double t = (dx * dx + dy * dy + dz * dz) * hinv2;
     const double mb = s.m[b];
     double w;
+    if (FAST) {
+      const fx::Vec3 D = vec64(dx, dy, dz, ed);
+      w = shape_at(fx::dot(D, D), 2 * (ed - 1023) - 60, hinv2);
+      acc += mb * w;
+      wrow[k] = w;
+      continue;
+    }
+    const double t = (dx * dx + dy * dy + dz * dz) * hinv2;
     if (GRADH) {
       double dw;
       if (sinc_n == 6)
@@ -150,13 +178,28 @@ __global__ void __launch_bounds__(kThreads64) k_iad64(const Grid* gp, StateView 
   const int cnt = valid ? min(L.nn[a], L.max_nb) : 0;
   const uint32_t* list = L.nbr + a * L.max_nb;
   const double* wrow = L.w + a * L.max_nb;
+  const int ed = fx::exp_above(2.0 * s.h[a]);  // |d| < 2 h_a
+  const bool mid = ed > 600 && ed < 1450;      // products stay normal
   double t00 = 0, t01 = 0, t02 = 0, t11 = 0, t12 = 0, t22 = 0;
   for (int k = sub; k < cnt; k += NSUB) {
     const int64_t b = entry_index(list[k]);
     double dx = s.x[b] - xa, dy = s.y[b] - ya, dz = s.z[b] - za;
     sep64(im, dx, dy, dz);
-    const double w = aux.vol[b] * wrow[k];
-    const double wx = w * dx, wy = w * dy, wz = w * dz;
+    // vol_b S^n d in fixed point (4 of 13 FP64 operations of a pair), in the
+    // middle of the exponent range
+    const double vol = aux.vol[b], sk = wrow[k];
+    double wx, wy, wz;
+    if (fx::middle(vol) && fx::middle(sk) && mid) {
+      const fx::Mant w = fx::mant(vol) * fx::mant(sk);
+      wx = fx::times(w, fx::fixed<61>(dx, ed), ed - 1023 - 61);
+      wy = fx::times(w, fx::fixed<61>(dy, ed), ed - 1023 - 61);
+      wz = fx::times(w, fx::fixed<61>(dz, ed), ed - 1023 - 61);
+    } else {
+      const double w = vol * sk;
+      wx = w * dx;
+      wy = w * dy;
+      wz = w * dz;
+    }
     t00 += wx * dx;
     t01 += wx * dy;
     t02 += wx * dz;
@@ -272,8 +315,11 @@ __device__ __forceinline__ void rows(const long long cf[6], fx::Vec3 R[3]) {
 // operations of a pair) are scalar products in block fixed point on the integer
 // pipes, d to the power of two above 2 h_a, v to its own: their rms error, about
 // 2^-60 of the largest components' product, is below FP64's.
-template <int NSUB>
-__global__ void __launch_bounds__(kThreads64) k_momentum64(const Grid* gp, const Rec64* rec,
+// FAST (exact kernel, n = 6): S^6 of the neighbour's kernel, its product with
+// m_b B_n/h_b^3 and x.v / r in fixed point too, except for pairs closer than
+// 1/16 of the power of two above 2 h_a, which need r^2 to FP64's relative precision.
+template <int NSUB, bool FAST>
+__global__ void __launch_bounds__(kThreads64, 4) k_momentum64(const Grid* gp, const Rec64* rec,
                                                            StateView s, OutView o, Aux64 aux,
                                                            Lists64 L, int64_t n, int sinc_n,
                                                            uint32_t* err) {
@@ -301,30 +347,37 @@ __global__ void __launch_bounds__(kThreads64) k_momentum64(const Grid* gp, const
     const Rec64* rb = rec + entry_index(list[k]);
     double dx = rb->x - xa, dy = rb->y - ya, dz = rb->z - za;
     sep64(im, dx, dy, dz);
-    const double r2 = dx * dx + dy * dy + dz * dz;
     const double vx = vxa - rb->vx, vy = vya - rb->vy, vz = vza - rb->vz;
-    fx::Vec3 D, V;
-    fx::put(D, 0, fx::fixed<61>(dx, ed));
-    fx::put(D, 1, fx::fixed<61>(dy, ed));
-    fx::put(D, 2, fx::fixed<61>(dz, ed));
+    const fx::Vec3 D = vec64(dx, dy, dz, ed);
     const int ev = max(fx::exp_above(vx), max(fx::exp_above(vy), fx::exp_above(vz)));
-    fx::put(V, 0, fx::fixed<61>(vx, ev));
-    fx::put(V, 1, fx::fixed<61>(vy, ev));
-    fx::put(V, 2, fx::fixed<61>(vz, ev));
+    const fx::Vec3 V = vec64(vx, vy, vz, ev);
     const double vnan = ev <= 2047 ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
     const int64_t vd = fx::dot(V, D);  // -x_ab . v_ab
+    const int kv = ev + ed - 2 * 1023 - 60, kr = 2 * (ed - 1023) - 60;
+    const int64_t R = FAST ? fx::dot(D, D) : 0;
+    double wv = 0.0, wb;  // x_ab . v_ab / r where negative
+    if (FAST && R >= (int64_t)1 << 52) {
+      uint64_t y;
+      wb = (uint64_t)R < (uint64_t)1 << 61 && fx::fraction_of((uint64_t)R, kr, rb->hinv2, y)
+               ? fx::S6_at_times(y, rb->mn) : 0.0;
+      if (vd > 0) wv = fx::over_root(-vd, kv, (uint64_t)R, kr);
+    } else {
+      const double r2 = dx * dx + dy * dy + dz * dz;
+      wb = rb->mn * shape64(r2 * rb->hinv2, sinc_n, aux.ktab);
+      if (vd > 0) {
+        double y0, e;
+        root_parts(r2, y0, e);
+        const double z = fx::scaled(-vd, kv) * y0;
+        wv = fma(z, e, z);
+      }
+    }
     double pa = 0.0, pb = 0.0;
     if (vd > 0) {
-      const double xv = fx::scaled(-vd, ev + ed - 2 * 1023 - 60);
-      double y0, e;
-      root_parts(r2, y0, e);
-      const double z = xv * y0, w = fma(z, e, z);
-      const double q = w * fma(3.0, w, -(ca + rb->c));
+      const double q = wv * fma(3.0, wv, -(ca + rb->c));
       pa = q * ira;
       pb = q * rb->irq;
     }
     const double wa = rb->m * wrow[k];
-    const double wb = rb->mn * shape64(r2 * rb->hinv2, sinc_n, aux.ktab);
     const double fa = wa * (Xa + pa);
     const double fb = wb * (rb->X + pb);
     {
@@ -400,6 +453,11 @@ inline Lists64 lists64_of(sph_ctx* ctx) {
   return t;
 }
 
+// The default kernel: exact, n = 6.
+inline bool fast64(const sph_ctx* ctx) {
+  return ctx->prm.kernel_mode == SPH_KERNEL_EXACT && ctx->prm.sinc_n == 6.0;
+}
+
 inline unsigned blocks64(int64_t n, int nsub) {
   return (unsigned)((n * nsub + kThreads64 - 1) / kThreads64);
 }
@@ -410,7 +468,9 @@ void launch_density_f64(sph_ctx* ctx, const StateView& s, const OutView& o, int6
                         cudaStream_t st) {
   with_lanes64(n, [&](auto lanes) {
     constexpr int NS = decltype(lanes)::value;
-    auto kern = ctx->prm.gradh ? k_density64<NS, true> : k_density64<NS, false>;
+    auto kern = ctx->prm.gradh ? k_density64<NS, true, false>
+                               : (fast64(ctx) ? k_density64<NS, false, true>
+                                              : k_density64<NS, false, false>);
     launch_dep(kern, blocks64(n, NS), kThreads64, 0, st, ctx->grid, s, o, aux_of(ctx),
         lists64_of(ctx), n, ctx->Bn, (int)ctx->prm.sinc_n, ctx->prm.gamma, ctx->prm.alpha,
         ctx->err);
@@ -437,7 +497,8 @@ void launch_momentum_f64(sph_ctx* ctx, const StateView& s, const OutView& o, int
   launch_dep(k_pack64, (unsigned)((n + 127) / 128), 128, 0, st, s, o, aux_of(ctx), n, rec);
   with_lanes64(n, [&](auto lanes) {
     constexpr int NS = decltype(lanes)::value;
-    launch_dep(k_momentum64<NS>, blocks64(n, NS), kThreads64, 0, st, ctx->grid, rec, s, o,
+    auto kern = fast64(ctx) ? k_momentum64<NS, true> : k_momentum64<NS, false>;
+    launch_dep(kern, blocks64(n, NS), kThreads64, 0, st, ctx->grid, rec, s, o,
         aux_of(ctx), lists64_of(ctx), n, (int)ctx->prm.sinc_n, ctx->err);
   });
   ctx->launches += 2;

@@ -42,6 +42,30 @@ extern "C" void dots(const double* a, const double* b, double* out, long n) {
     out[i] = scaled(dot(A, B), ea + eb - 2 * 1023 - 59);
   }
 }
+// for d (3 per entry), 2 h_a, 1 / h_b^2, v, a: S^6 at t = r^2 / h_b^2, its product with a, v.d / r
+// (0 where r is below 1/16 of the power of two above 2 h_a), and (a S^6) d_x
+extern "C" void pair(const double* d, const double* h2, const double* hinv2, const double* v,
+                     const double* a, double* out, long n) {
+  using namespace sph::fx;
+  for (long i = 0; i < n; ++i, d += 3, v += 3, out += 4) {
+    const int ed = exp_above(h2[i]), kr = 2 * (ed - 1023) - 60;
+    int ev = 1;
+    for (int k = 0; k < 3; ++k) if (exp_above(v[k]) > ev) ev = exp_above(v[k]);
+    Vec3 D, V;
+    for (int k = 0; k < 3; ++k) {
+      put(D, k, fixed<61>(d[k], ed));
+      put(V, k, fixed<61>(v[k], ev));
+    }
+    const int64_t R = dot(D, D), vd = dot(V, D);
+    uint64_t y;
+    const bool in = (uint64_t)R >> 60 == 0 && fraction_of((uint64_t)R, kr, hinv2[i], y);
+    out[0] = in ? S6_at(y) : 0.0;
+    out[1] = in ? S6_at_times(y, a[i]) : 0.0;
+    out[2] = R >> 52 && vd ? over_root(vd, ev + ed - 2 * 1023 - 60, (uint64_t)R, kr) : 0.0;
+    out[3] = middle(a[i]) && middle(out[0])
+                 ? times(mant(a[i]) * mant(out[0]), fixed<61>(d[0], ed), ed - 1023 - 61) : 0.0;
+  }
+}
 """
 
 
@@ -58,6 +82,11 @@ def fixed(tmp_path_factory):
         if b is not None:
             out = np.empty(len(t))
             f.dots(*[v.ctypes.data_as(C.c_void_p) for v in (t, b, out)], C.c_long(len(t)))
+            return out
+        if isinstance(t, tuple):
+            out = np.empty((len(t[1]), 4))
+            f.pair(*[np.ascontiguousarray(v).ctypes.data_as(C.c_void_p) for v in t],
+                   out.ctypes.data_as(C.c_void_p), C.c_long(len(t[1])))
             return out
         t = np.ascontiguousarray(t, dtype=np.float64)
         out = [np.empty_like(t) for _ in range(3)]
@@ -131,6 +160,48 @@ def test_block_fixed_point_dot(fixed):
         assert abs(Fraction(v) - exact) <= bound + abs(exact) / 2 ** 53, (x, y, v)
 
 
+def test_pair_in_fixed_point(fixed):
+    """The pair quantities the FP64 kernels take from block fixed point, against mpmath.  R carries
+    an error of at most 3.5 units of 2^-60 of 2^(2 e) (2^e the power of two above 2 h_a) plus the
+    truncation of d (6 units of 2^-61 times |d| / 2^e <= 1): 7 units together; y = R K 2^-60 with
+    K = 2^(2e) / (4 h_b^2), plus 2^-57.  |dS^6/dy| <= 10."""
+    mp = pytest.importorskip("mpmath")
+    mp.mp.dps = 40
+    rng = np.random.default_rng(3)
+    n = 600
+    h = 2.0 ** rng.uniform(-30, 30, n)
+    hb = h * 2.0 ** rng.uniform(-0.7, 0.7, n)
+    hb[::29] = h[::29] * 4.0
+    u = rng.normal(size=(n, 3))
+    r = 2 * h * rng.uniform(0, 1, n) ** (1 / 3)
+    r[::13] *= 1e-3
+    d = u / np.linalg.norm(u, axis=1)[:, None] * r[:, None] * (1 - 1e-12)
+    v = rng.normal(size=(n, 3)) * 2.0 ** rng.uniform(-40, 40, (n, 1))
+    a = 2.0 ** rng.uniform(-90, 90, n)
+    hinv2 = 1.0 / (hb * hb)
+    out = fixed((d, 2 * h, hinv2, v, a))
+    for i in range(n):
+        D, V = [mp.mpf(x) for x in d[i]], [mp.mpf(x) for x in v[i]]
+        r2 = sum(x * x for x in D)
+        t = r2 * mp.mpf(hinv2[i])
+        x = mp.pi / 2 * mp.sqrt(t)
+        S6 = (mp.sin(x) / x) ** 6 if t < 4 else mp.mpf(0)
+        top = 2.0 ** np.frexp(2 * h[i])[1]
+        err = 10 * (7 * 2.0 ** -60 * top * top * hinv2[i] / 4 + 2.0 ** -57) + 2.0 ** -52 * S6
+        assert abs(out[i, 0] - S6) <= err, i
+        assert abs(out[i, 1] - a[i] * S6) <= a[i] * (err + 2.0 ** -52 * S6), i
+        if out[i, 2]:
+            vd = sum(p * q for p, q in zip(V, D))
+            vtop = 2.0 ** np.frexp(np.abs(v[i]).max())[1]
+            # v.d to 9.5 units of 2^-60, 1/r to 7 units of 2^-60 of top^2 / r^2 (halved), rounding
+            tol = (9.5 * 2.0 ** -60 * vtop * top / mp.sqrt(r2)
+                   + abs(vd) / mp.sqrt(r2) * (3.5 * 2.0 ** -60 * top * top / r2 + 2.0 ** -52))
+            assert abs(out[i, 2] - vd / mp.sqrt(r2)) <= tol, i
+        if out[i, 3]:
+            e = mp.mpf(a[i]) * mp.mpf(out[i, 0]) * D[0]
+            assert abs(out[i, 3] - e) <= a[i] * out[i, 0] * top * 2.0 ** -60 + 2.0 ** -52 * abs(e), i
+
+
 # particles per target-lane split: 16 lanes (below 16,384), 8, 4 (from 131,072)
 @pytest.mark.gpu
 @pytest.mark.parametrize("side,gradh", [(7, 0), (25, 1), (26, 0), (50, 0), (51, 1)])
@@ -175,3 +246,34 @@ def test_gravity_scales(side, scale, precision, tol):
     ref = ref[np.argsort(s["id"])]
     assert np.abs(g[np.argsort(ids)] - ref).max() <= tol * np.abs(ref).max()
     np.testing.assert_array_equal(counts, st)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("opts", [{}, {"sinc_n": 5.0}, {"gradh": 1}, {"kernel_mode": "table"}])
+def test_fp64_close_pairs_and_uneven_h(opts):
+    """Pairs at 1e-2 to 1e-9 of h (below the range where r is taken from fixed point), smoothing
+    lengths over a factor of 4, one axis at rest, and every kernel form, against the oracle."""
+    from paper_2005_02656_gb300 import SphSim
+    s = sph_inputs.jittered_box(14, seed_index=77)
+    rng = np.random.default_rng(8)
+    n = s["x"].shape[0]
+    s["h"] = s["h"] * np.exp(rng.uniform(-0.7, 0.6, n))
+    for k, f in enumerate((1e-2, 1e-4, 1e-6, 1e-9)):
+        i, j = 50 + 2 * k, 51 + 2 * k
+        for ax, c in zip("xyz", (1.0, -0.5, 0.25)):
+            s[ax][j] = s[ax][i] + c * f * s["h"][i]
+    s["vz"][:] = 0.0
+    kw = {k: (1 if v == "table" else v) for k, v in opts.items()}
+    rc, _, ref = oracle_outputs(s, ng_target=0, max_nb=800, **kw)
+    assert rc == 0
+    sim = SphSim(s, ng_target=0, max_nb=800, **opts)
+    sim.find_neighbors()
+    sim.density()
+    sim.iad()
+    sim.momentum_energy()
+    got = sim.to_numpy()
+    assert sim.error_word() == 0
+    sim.close()
+    e = field_errors(got, ref)
+    for k in ("rho", "p", "c", "iad", "a", "du"):
+        assert e[k] <= 1e-12, (k, e)
