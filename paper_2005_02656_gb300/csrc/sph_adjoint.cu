@@ -217,15 +217,19 @@ __global__ void k_adj_prep(Slot sl, Prep pr, int64_t n, double Bn, int gradh) {
 
 // ---------------------------------------------------------------------------
 // Reverse of update + momentum/energy, the target's side.  The FP64 pipe bounds
-// the kernel: about 180 operations per pair, the kernel values and their
-// derivatives taken from the fixed-point series (sph_fixed.cuh) and the partials
-// built from the scalars g.C_a d, v.C_a d and so on instead of the vectors A.
-// 64,000 particles, FP64 series and comparisons and one thread per target before:
-// 4.19 -> 2.40 ms (IAD 1.22 -> 0.79, neighbour side 0.54 -> 0.45, density 0.57 ->
-// 0.34 ms by the integer minimum image and the split over lanes).
+// the kernel (74% of its cycles, the rest latency with twelve warps per SM), so
+// the partials are built from the scalars g.C_a d, v.C_a d and so on instead of
+// the vectors A, and every scalar product of a pair is block fixed point on the
+// integer pipes; FAST (n = 6): kernel values, their derivatives and 1/r as well,
+// from r^2 in fixed point (sph_fixed.cuh).  About 120 FP64 operations per pair
+// are left.  64,000 particles: 1.95 ms, 2.40 with FP64 products, 4.19 with the
+// FP64 series and one thread per target (IAD 1.22 -> 0.79, neighbour side 0.54 ->
+// 0.45, density 0.57 -> 0.34 ms by the integer minimum image and the split over
+// lanes).  168 registers for a third CTA with 330 bytes spilled: 5% under two CTAs
+// without spills; four CTAs: no gain, 700 bytes.
 // ---------------------------------------------------------------------------
-template <int NSUB>
-__global__ void __launch_bounds__(kThreads) k_adj_momentum_a(Slot sl, Prep pr, Bar q, Work w,
+template <int NSUB, bool FAST>
+__global__ void __launch_bounds__(kThreads, 3) k_adj_momentum_a(Slot sl, Prep pr, Bar q, Work w,
                                                              PairBuf pb, int64_t n, Consts kc,
                                                              double* apart) {
   constexpr int kT = kThreads / NSUB;  // targets of a block
@@ -262,9 +266,15 @@ __global__ void __launch_bounds__(kThreads) k_adj_momentum_a(Slot sl, Prep pr, B
     const double ira = pr.ir[a];
     const double Xa = pr.X[a];
     const double ca = sl.c[a];
-    double Ca[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) Ca[i] = sl.iad[6 * a + i];
+    const int ed = sph::fx::exp_above(2.0 * s.h[a]);  // |d| < 2 h_a
+    const int eg = sph::exp_above3(gx, gy, gz);
+    const sph::fx::Vec3 Gv = sph::vec64(gx, gy, gz, eg);
+    long long cf[6];
+    const int eca = sph::fix_matrix(sl.iad + 6 * a, cf);
+    sph::fx::Vec3 Ca[3];
+    sph::rows(cf, Ca);
+    // NaN where a matrix or g is not finite (their fixed-point forms are not)
+    const double nan_a = eca == 0 || eg > 2047 ? __longlong_as_double(0x7ff8000000000000LL) : 0.0;
     double xbx = 0, xby = 0, xbz = 0, vbx = 0, vby = 0, vbz = 0;
     double Xbar = 0, irbar = 0, cbar = 0;
     double Cbar[6] = {0, 0, 0, 0, 0, 0};
@@ -274,33 +284,63 @@ __global__ void __launch_bounds__(kThreads) k_adj_momentum_a(Slot sl, Prep pr, B
       const int64_t b = sph::entry_index(list[k]);
       double dx = s.x[b] - xa, dy = s.y[b] - ya, dz = s.z[b] - za;
       sep64(im, dx, dy, dz);
-      const double r2 = dx * dx + dy * dy + dz * dz;
+      const double vabx = vxa - s.vx[b], vaby = vya - s.vy[b], vabz = vza - s.vz[b];
+      const sph::fx::Vec3 D = sph::vec64(dx, dy, dz, ed);
+      const int ev = sph::exp_above3(vabx, vaby, vabz);
+      const sph::fx::Vec3 V = sph::vec64(vabx, vaby, vabz, ev);
+      const int64_t vd = sph::fx::dot(V, D);  // -x_ab . v_ab
+      const int kr = 2 * (ed - 1023) - 60;
+      const int64_t R = FAST ? sph::fx::dot(D, D) : 0;
+      const bool on = vd > 0;
+      const double hinv2b = pr.hinv2[b], normb = pr.norm[b];
       double Wa, dWa, Wb, dWb;  // W and dW / d r^2
-      shape_d(r2 * hinv2a, kc.sinc_n, Wa, dWa);
+      double rinv = 0.0;
+      if (FAST && R >= (int64_t)1 << 52) {
+        uint64_t y;
+        Wa = dWa = Wb = dWb = 0.0;
+        const bool in = (uint64_t)R >> 60 == 0;
+        if (in && sph::fx::fraction_of((uint64_t)R, kr, hinv2a, y)) sph::fx::S6_d_at(y, Wa, dWa);
+        if ((uint64_t)R >> 61 == 0 && sph::fx::fraction_of((uint64_t)R, kr, hinv2b, y))
+          sph::fx::S6_d_at(y, Wb, dWb);
+        if (on) rinv = sph::fx::over_root((int64_t)1 << 60, -60, (uint64_t)R, kr);
+      } else {
+        const double r2 = dx * dx + dy * dy + dz * dz;
+        shape_d(r2 * hinv2a, kc.sinc_n, Wa, dWa);
+        const double tb = r2 * hinv2b;
+        Wb = dWb = 0.0;
+        if (__double2hiint(tb) < 0x40100000) shape_d(tb, kc.sinc_n, Wb, dWb);  // t_b < 4
+        if (on) rinv = sph::inv_root(r2);
+      }
       Wa *= norma;
       dWa *= dnorma;
-      const double hinv2b = pr.hinv2[b], normb = pr.norm[b];
-      const double tb = r2 * hinv2b;
-      Wb = dWb = 0.0;
-      if (__double2hiint(tb) < 0x40100000) shape_d(tb, kc.sinc_n, Wb, dWb);  // t_b < 4
       Wb *= normb;
       dWb *= normb * hinv2b;
-      double Cb[6];
+      sph::fx::Vec3 Cb[3], Ua, Ub;
+      const int ecb = sph::fix_matrix(sl.iad + 6 * b, cf);
+      sph::rows(cf, Cb);
+      // C_a d and C_b d, and their products with g and v
+      const int ka = eca + ed - 2 * 1023 - 59, kb = ecb + ed - 2 * 1023 - 59;
+      double ca_[3], cb_[3];
 #pragma unroll
-      for (int i = 0; i < 6; ++i) Cb[i] = sl.iad[6 * b + i];
-      double cax, cay, caz, cbx, cby, cbz;
-      sym_mv(Ca, dx, dy, dz, cax, cay, caz);
-      sym_mv(Cb, dx, dy, dz, cbx, cby, cbz);
-      const double vabx = vxa - s.vx[b], vaby = vya - s.vy[b], vabz = vza - s.vz[b];
-      const double xv = -(dx * vabx + dy * vaby + dz * vabz);
+      for (int i = 0; i < 3; ++i) {
+        const int64_t ua = sph::fx::dot(Ca[i], D), ub = sph::fx::dot(Cb[i], D);
+        sph::fx::put(Ua, i, ua);
+        sph::fx::put(Ub, i, ub);
+        ca_[i] = sph::fx::scaled(ua, ka);
+        cb_[i] = sph::fx::scaled(ub, kb);
+      }
+      const double cax = ca_[0], cay = ca_[1], caz = ca_[2];
+      const double cbx = cb_[0], cby = cb_[1], cbz = cb_[2];
+      const double gca = sph::fx::scaled(sph::fx::dot(Gv, Ua), ka + eg - 1023 + 1);
+      const double gcb = sph::fx::scaled(sph::fx::dot(Gv, Ub), kb + eg - 1023 + 1);
+      const double vca = sph::fx::scaled(sph::fx::dot(V, Ua), ka + ev - 1023 + 1);
+      const double vcb = sph::fx::scaled(sph::fx::dot(V, Ub), kb + ev - 1023 + 1);
       const double irb = pr.ir[b];
       const double Xb = pr.X[b];
       const double cab = ca + sl.c[b];
-      const bool on = sph::okey(xv, 0) < 0;  // xv < 0
-      double rinv = 0.0, wv = 0.0, vsig = 0.0, hPi = 0.0;  // hPi = Pi / 2
+      double wv = 0.0, vsig = 0.0, hPi = 0.0;  // hPi = Pi / 2
       if (on) {
-        rinv = sph::inv_root(r2);
-        wv = xv * rinv;
+        wv = sph::fx::scaled(-vd, ev + ed - 2 * 1023 - 60) * rinv;
         vsig = cab - 3.0 * wv;
         hPi = 0.5 * mha * vsig * wv;
       }
@@ -309,10 +349,6 @@ __global__ void __launch_bounds__(kThreads) k_adj_momentum_a(Slot sl, Prep pr, B
       // partials of L_pair = -m_b (fa1 g.A_a + fb1 g.A_b) + e m_b (fa2 v.A_a + fb2 v.A_b),
       // fa1 = X_a + p_a, fb1 = X_b + p_b, fa2 = X_a + p_a / 2, fb2 = p_b / 2,
       // A_a = W_a C_a d, A_b = W_b C_b d
-      const double gca = gx * cax + gy * cay + gz * caz;
-      const double gcb = gx * cbx + gy * cby + gz * cbz;
-      const double vca = vabx * cax + vaby * cay + vabz * caz;
-      const double vcb = vabx * cbx + vaby * cby + vabz * cbz;
       const double emb = e * mb_;
       const double ma_w = mb_ * Wa, mb_w = mb_ * Wb;
       const double fa1b = -ma_w * gca, fb1b = -mb_w * gcb;
@@ -339,12 +375,19 @@ __global__ void __launch_bounds__(kThreads) k_adj_momentum_a(Slot sl, Prep pr, B
       Cbar[3] += say * dy;
       Cbar[4] += say * dz + saz * dy;
       Cbar[5] += saz * dz;
-      double dbx = Ca[0] * sax + Ca[1] * say + Ca[2] * saz;
-      double dby = Ca[1] * sax + Ca[3] * say + Ca[4] * saz;
-      double dbz = Ca[2] * sax + Ca[4] * say + Ca[5] * saz;
-      dbx += Cb[0] * sbx + Cb[1] * sby + Cb[2] * sbz;
-      dby += Cb[1] * sbx + Cb[3] * sby + Cb[4] * sbz;
-      dbz += Cb[2] * sbx + Cb[4] * sby + Cb[5] * sbz;
+      // C_a s_a + C_b s_b
+      const int esa = sph::exp_above3(sax, say, saz), esb = sph::exp_above3(sbx, sby, sbz);
+      const sph::fx::Vec3 Sa = sph::vec64(sax, say, saz, esa), Sb = sph::vec64(sbx, sby, sbz, esb);
+      const int kas = eca + esa - 2 * 1023 - 59, kbs = ecb + esb - 2 * 1023 - 59;
+      double dbx = sph::fx::scaled(sph::fx::dot(Ca[0], Sa), kas) +
+                   sph::fx::scaled(sph::fx::dot(Cb[0], Sb), kbs);
+      double dby = sph::fx::scaled(sph::fx::dot(Ca[1], Sa), kas) +
+                   sph::fx::scaled(sph::fx::dot(Cb[1], Sb), kbs);
+      double dbz = sph::fx::scaled(sph::fx::dot(Ca[2], Sa), kas) +
+                   sph::fx::scaled(sph::fx::dot(Cb[2], Sb), kbs);
+      // a value that is not finite has no fixed-point form: NaN instead
+      if (max(max(ev, ecb == 0 ? 2048 : 0), max(esa, esb)) > 2047)
+        dbx = __longlong_as_double(0x7ff8000000000000LL);
       double r2b = (Pa * gca + Qa * vca) * dWa + (Pb * gcb + Qb * vcb) * dWb;
       double cpair = 0.0;
       if (on) {
@@ -381,7 +424,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_momentum_a(Slot sl, Prep pr, B
       rec[5] = make_double2(sby, sbz);
       pb.wk[slot] = make_double2(Wa, dWa);
     }
-    lanes_sum<NSUB>(xbx, sums[0]);
+    lanes_sum<NSUB>(xbx + nan_a, sums[0]);
     lanes_sum<NSUB>(xby, sums[1]);
     lanes_sum<NSUB>(xbz, sums[2]);
     lanes_sum<NSUB>(vbx, sums[3]);
@@ -1068,7 +1111,8 @@ int reverse_step(sph_adj* A, int j, cudaStream_t st) {
     constexpr int NS = decltype(lanes)::value;
     const unsigned gl = (unsigned)((n * NS + kThreads - 1) / kThreads);
     const unsigned ga = gl < kAlphaBlocks ? gl : kAlphaBlocks;
-    k_adj_momentum_a<NS><<<ga, kThreads, 0, st>>>(sl, A->pr, A->q, A->w, A->pb, n, kc, A->apart);
+    auto momentum_a = kc.sinc_n == 6 ? k_adj_momentum_a<NS, true> : k_adj_momentum_a<NS, false>;
+    momentum_a<<<ga, kThreads, 0, st>>>(sl, A->pr, A->q, A->w, A->pb, n, kc, A->apart);
     k_alpha_sum<<<1, 1024, 0, st>>>(A->apart, (int)ga, A->alpha_acc);
     k_adj_momentum_b<NS><<<gl, kThreads, 0, st>>>(sl, A->w, A->pb, rev_of(A), n, kc);
     k_adj_iad<NS><<<gl, kThreads, 0, st>>>(sl, A->pr, A->w, A->pb, rev_of(A), n, kc);

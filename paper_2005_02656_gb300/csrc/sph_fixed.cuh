@@ -152,11 +152,10 @@ SPH_FX double S6_at_times(uint64_t y, double a) {
   return from_bits(bits_of(pack(f, 6 - 6 * z + E - 1022)) | (b & 0x8000000000000000u));
 }
 
-// S^6 and its derivative by t, 6 S^5 dS/dt (dS/dt = (dS/dy) / 4).
-SPH_FX void S6_d(double t, double& w, double& dw) {
+// S^6 and its derivative by t, 6 S^5 dS/dt (dS/dt = (dS/dy) / 4), at the
+// fraction y = t / 4.
+SPH_FX void S6_d_at(uint64_t y, double& w, double& dw) {
   w = dw = 0.0;
-  if ((uint32_t)(bits_of(t) >> 32) >= 0x40100000u) return;
-  const uint64_t y = fraction(t);
   const uint64_t s = sinc(y);
   if (s == 0) return;
   const int z = clz64(s);
@@ -166,6 +165,10 @@ SPH_FX void S6_d(double t, double& w, double& dw) {
   // 1.5 S^5 D: D in units of 2^-63 and 1.5 = 0.75 * 2 add two to the exponent
   const uint64_t d = mulhi64(mulhi64(m4, m), sinc_slope(y));
   dw = -pack(d - (d >> 2), 7 - 5 * z);
+}
+SPH_FX void S6_d(double t, double& w, double& dw) {
+  w = dw = 0.0;
+  if ((uint32_t)(bits_of(t) >> 32) < 0x40100000u) S6_d_at(fraction(t), w, dw);
 }
 
 // --- vectors in block fixed point ---

@@ -1,11 +1,13 @@
 // What the FP64 pair kernels (sph_pairs_fp64.cu) and their reverse kernels
-// (sph_adjoint.cu) share: the minimum image decided on the integer pipes, and
-// the split of a target's neighbours over lanes.
+// (sph_adjoint.cu) share: the minimum image decided on the integer pipes,
+// vectors and matrices in block fixed point, and the split of a target's
+// neighbours over lanes.
 #pragma once
 
 #include <type_traits>
 
 #include "sph_device.cuh"
+#include "sph_fixed.cuh"
 #include "sph_internal.cuh"
 
 namespace sph {
@@ -42,6 +44,46 @@ __device__ __forceinline__ void sep64(const Image64& im, double& dx, double& dy,
     if (fy) dy += __double2hiint(dy) < 0 ? im.L[1] : -im.L[1];
     if (fz) dz += __double2hiint(dz) < 0 ? im.L[2] : -im.L[2];
   }
+}
+
+// Power of two above three components (fx::exp_above; over 2047: not finite).
+__device__ __forceinline__ int exp_above3(double x, double y, double z) {
+  return max(fx::exp_above(x), max(fx::exp_above(y), fx::exp_above(z)));
+}
+
+// A vector in block fixed point with the given power of two.
+__device__ __forceinline__ fx::Vec3 vec64(double x, double y, double z, int eb) {
+  fx::Vec3 v;
+  fx::put(v, 0, fx::fixed<61>(x, eb));
+  fx::put(v, 1, fx::fixed<61>(y, eb));
+  fx::put(v, 2, fx::fixed<61>(z, eb));
+  return v;
+}
+
+// C (6 entries) as block fixed point; the exponent field of the power of two
+// above its largest entry, or 0 where an entry is not finite.
+__device__ __forceinline__ int fix_matrix(const double* C, long long cf[6]) {
+  int eb = 1;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) eb = max(eb, fx::exp_above(C[q]));
+#pragma unroll
+  for (int q = 0; q < 6; ++q) cf[q] = fx::fixed<60>(C[q], eb);
+  return eb <= 2047 ? eb : 0;
+}
+
+// 2^(eb - 1023) for eb of fix_matrix (not finite: NaN).
+__device__ __forceinline__ double power_of(int eb) {
+  if (eb == 0) return __longlong_as_double(0x7ff8000000000000LL);
+  return eb < 2047 ? __hiloint2double(eb << 20, 0) : 2.0 * __hiloint2double(2046 << 20, 0);
+}
+
+// Rows of a symmetric matrix in block fixed point.
+__device__ __forceinline__ void rows(const long long cf[6], fx::Vec3 R[3]) {
+  constexpr int at[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) fx::put(R[i], j, cf[at[i][j]]);
 }
 
 // Sum over the NSUB lanes of a target, left in sums[target of the block].

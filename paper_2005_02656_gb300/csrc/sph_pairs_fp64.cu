@@ -58,15 +58,6 @@ __device__ __forceinline__ double shape64(double t, int n, const double2* tab) {
   return n == 6 ? fx::S6(t) : ipow(fx::S(t), n);
 }
 
-// A vector in block fixed point with the given power of two.
-__device__ __forceinline__ fx::Vec3 vec64(double x, double y, double z, int eb) {
-  fx::Vec3 v;
-  fx::put(v, 0, fx::fixed<61>(x, eb));
-  fx::put(v, 1, fx::fixed<61>(y, eb));
-  fx::put(v, 2, fx::fixed<61>(z, eb));
-  return v;
-}
-
 // S^6 of r^2 = R 2^k and 1 / h^2; 0 from the support's edge on (R reaches 2^60 at
 // the target's own).
 __device__ __forceinline__ double shape_at(int64_t R, int k, double hinv2) {
@@ -258,23 +249,6 @@ struct alignas(16) Rec64 {
   long long cf[6];   // C in block fixed point (fx::fixed), xx xy xz yy yz zz
 };
 
-// C (6 entries) as block fixed point; the exponent field of the power of two
-// above its largest entry, or 0 where an entry is not finite.
-__device__ __forceinline__ int fix_matrix(const double* C, long long cf[6]) {
-  int eb = 1;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) eb = max(eb, fx::exp_above(C[q]));
-#pragma unroll
-  for (int q = 0; q < 6; ++q) cf[q] = fx::fixed<60>(C[q], eb);
-  return eb <= 2047 ? eb : 0;
-}
-
-// 2^(eb - 1023) for eb of fix_matrix (not finite: NaN).
-__device__ __forceinline__ double power_of(int eb) {
-  if (eb == 0) return __longlong_as_double(0x7ff8000000000000LL);
-  return eb < 2047 ? __hiloint2double(eb << 20, 0) : 2.0 * __hiloint2double(2046 << 20, 0);
-}
-
 __global__ void k_pack64(StateView s, OutView o, Aux64 aux, int64_t n, Rec64* rec) {
   dep_enter();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -296,15 +270,6 @@ __global__ void k_pack64(StateView s, OutView o, Aux64 aux, int64_t n, Rec64* re
   for (int q = 0; q < 6; ++q) C[q] = o.iad[6 * i + q];
   r.mn = aux.mn[i] * power_of(fix_matrix(C, r.cf));
   rec[i] = r;
-}
-
-// Rows of a symmetric matrix in block fixed point.
-__device__ __forceinline__ void rows(const long long cf[6], fx::Vec3 R[3]) {
-  constexpr int at[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) fx::put(R[i], j, cf[at[i][j]]);
 }
 
 // Per pair, with p_a = Pi / (2 rho_a) and p_b = Pi / (2 rho_b):
@@ -349,7 +314,7 @@ __global__ void __launch_bounds__(kThreads64, 4) k_momentum64(const Grid* gp, co
     sep64(im, dx, dy, dz);
     const double vx = vxa - rb->vx, vy = vya - rb->vy, vz = vza - rb->vz;
     const fx::Vec3 D = vec64(dx, dy, dz, ed);
-    const int ev = max(fx::exp_above(vx), max(fx::exp_above(vy), fx::exp_above(vz)));
+    const int ev = exp_above3(vx, vy, vz);
     const fx::Vec3 V = vec64(vx, vy, vz, ev);
     const double vnan = ev <= 2047 ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
     const int64_t vd = fx::dot(V, D);  // -x_ab . v_ab
