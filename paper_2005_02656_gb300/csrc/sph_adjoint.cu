@@ -128,34 +128,32 @@ __device__ __forceinline__ void shape_d(double t, int n, double& w, double& dw) 
     sph::kernel_w64_d(t, 1.0, n, w, dw);
 }
 
-// y = C x for C stored as (xx, xy, xz, yy, yz, zz).
-__device__ __forceinline__ void sym_mv(const double* C, double x0, double x1, double x2,
-                                       double& y0, double& y1, double& y2) {
-  y0 = C[0] * x0 + C[1] * x1 + C[2] * x2;
-  y1 = C[1] * x0 + C[3] * x1 + C[4] * x2;
-  y2 = C[2] * x0 + C[4] * x1 + C[5] * x2;
-}
-
 // ---------------------------------------------------------------------------
 // Reverse lists
 // ---------------------------------------------------------------------------
+// A warp per row: the row's atomics in flight at once (a thread per row took 48
+// and 99 us at 64,000 particles, 33 and 60 now).
 __global__ void k_rev_count(const int32_t* nn, const uint32_t* nbr, int mb, int64_t n,
                             int32_t* cnt) {
-  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n;
-       a += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t a = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); a < n;
+       a += step) {
     const int c = min(nn[a], mb);
     const uint32_t* row = nbr + a * mb;
-    for (int k = 0; k < c; ++k) atomicAdd(&cnt[sph::entry_index(row[k])], 1);
+    for (int k = lane; k < c; k += 32) atomicAdd(&cnt[sph::entry_index(row[k])], 1);
   }
 }
 
 __global__ void k_rev_fill(const int32_t* nn, const uint32_t* nbr, int mb, int64_t n,
                            const int64_t* start, int32_t* fill, uint64_t* list) {
-  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n;
-       a += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t a = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); a < n;
+       a += step) {
     const int c = min(nn[a], mb);
     const uint32_t* row = nbr + a * mb;
-    for (int k = 0; k < c; ++k) {
+    for (int k = lane; k < c; k += 32) {
       const int b = sph::entry_index(row[k]);
       const int pos = atomicAdd(&fill[b], 1);
       list[start[b] + pos] = ((uint64_t)a << kKBits) | (uint64_t)k;
@@ -164,11 +162,13 @@ __global__ void k_rev_fill(const int32_t* nn, const uint32_t* nbr, int mb, int64
 }
 
 // Sorts every row ascending: a warp per row, rank of each entry among the
-// row's (distinct) entries; rows longer than kRowSmem by one lane's
-// insertion sort in place.
+// row's entries, whose a are distinct and below 2^31 (a list holds a particle
+// once); rows longer than kRowSmem by one lane's insertion sort in place.  The
+// integer pipes bound it, so a rank is taken on the a alone and four entries of a
+// lane share a read of the row (64,000 particles: 134 us on whole entries, 106 now).
 __global__ void __launch_bounds__(kSortWarps * 32) k_rev_sort(const int64_t* start, int64_t n,
                                                               uint64_t* list) {
-  __shared__ uint64_t buf[kSortWarps][kRowSmem];
+  __shared__ uint32_t buf[kSortWarps][kRowSmem];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int64_t b = blockIdx.x * (int64_t)kSortWarps + w; b < n;
        b += (int64_t)gridDim.x * kSortWarps) {
@@ -177,13 +177,32 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_rev_sort(const int64_t* sta
     if (L <= 1) continue;
     uint64_t* row = list + s0;
     if (L <= kRowSmem) {
-      for (int i = lane; i < L; i += 32) buf[w][i] = row[i];
+      // up to four entries of a lane at a time; the row is written when all are read
+      uint64_t e[kRowSmem / 32];
+#pragma unroll
+      for (int g = 0; g < kRowSmem / 32; ++g)
+        if (32 * g < L) {
+          const int i = 32 * g + lane;
+          e[g] = i < L ? row[i] : ~(uint64_t)0;
+          if (i < L) buf[w][i] = (uint32_t)(e[g] >> kKBits);
+        }
       __syncwarp();
-      for (int i = lane; i < L; i += 32) {
-        const uint64_t e = buf[w][i];
-        int rank = 0;
-        for (int j = 0; j < L; ++j) rank += buf[w][j] < e;
-        row[rank] = e;
+#pragma unroll
+      for (int g = 0; g < kRowSmem / 32; g += 4) {
+        if (32 * g < L) {
+          uint32_t key[4];
+          int rank[4] = {0, 0, 0, 0};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) key[q] = (uint32_t)(e[g + q] >> kKBits);
+          for (int j = 0; j < L; ++j) {
+            const uint32_t v = buf[w][j];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) rank[q] += v < key[q];
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (32 * (g + q) + lane < L) row[rank[q]] = e[g + q];
+        }
       }
       __syncwarp();
     } else if (lane == 0) {
@@ -223,8 +242,8 @@ __global__ void k_adj_prep(Slot sl, Prep pr, int64_t n, double Bn, int gradh) {
 // integer pipes; FAST (n = 6): kernel values, their derivatives and 1/r as well,
 // from r^2 in fixed point (sph_fixed.cuh).  About 120 FP64 operations per pair
 // are left.  64,000 particles: 1.95 ms, 2.40 with FP64 products, 4.19 with the
-// FP64 series and one thread per target (IAD 1.22 -> 0.79, neighbour side 0.54 ->
-// 0.45, density 0.57 -> 0.34 ms by the integer minimum image and the split over
+// FP64 series and one thread per target (neighbour side 0.54 -> 0.45,
+// density 0.57 -> 0.34 ms by the integer minimum image and the split over
 // lanes).  168 registers for a third CTA with 330 bytes spilled: 5% under two CTAs
 // without spills; four CTAs: no gain, 700 bytes.
 // ---------------------------------------------------------------------------
@@ -326,21 +345,21 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_momentum_a(Slot sl, Prep pr
         const int64_t ua = sph::fx::dot(Ca[i], D), ub = sph::fx::dot(Cb[i], D);
         sph::fx::put(Ua, i, ua);
         sph::fx::put(Ub, i, ub);
-        ca_[i] = sph::fx::scaled(ua, ka);
-        cb_[i] = sph::fx::scaled(ub, kb);
+        ca_[i] = sph::fx::scaled<true>(ua, ka);
+        cb_[i] = sph::fx::scaled<true>(ub, kb);
       }
       const double cax = ca_[0], cay = ca_[1], caz = ca_[2];
       const double cbx = cb_[0], cby = cb_[1], cbz = cb_[2];
-      const double gca = sph::fx::scaled(sph::fx::dot(Gv, Ua), ka + eg - 1023 + 1);
-      const double gcb = sph::fx::scaled(sph::fx::dot(Gv, Ub), kb + eg - 1023 + 1);
-      const double vca = sph::fx::scaled(sph::fx::dot(V, Ua), ka + ev - 1023 + 1);
-      const double vcb = sph::fx::scaled(sph::fx::dot(V, Ub), kb + ev - 1023 + 1);
+      const double gca = sph::fx::scaled<true>(sph::fx::dot(Gv, Ua), ka + eg - 1023 + 1);
+      const double gcb = sph::fx::scaled<true>(sph::fx::dot(Gv, Ub), kb + eg - 1023 + 1);
+      const double vca = sph::fx::scaled<true>(sph::fx::dot(V, Ua), ka + ev - 1023 + 1);
+      const double vcb = sph::fx::scaled<true>(sph::fx::dot(V, Ub), kb + ev - 1023 + 1);
       const double irb = pr.ir[b];
       const double Xb = pr.X[b];
       const double cab = ca + sl.c[b];
       double wv = 0.0, vsig = 0.0, hPi = 0.0;  // hPi = Pi / 2
       if (on) {
-        wv = sph::fx::scaled(-vd, ev + ed - 2 * 1023 - 60) * rinv;
+        wv = sph::fx::scaled<true>(-vd, ev + ed - 2 * 1023 - 60) * rinv;
         vsig = cab - 3.0 * wv;
         hPi = 0.5 * mha * vsig * wv;
       }
@@ -379,12 +398,12 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_momentum_a(Slot sl, Prep pr
       const int esa = sph::exp_above3(sax, say, saz), esb = sph::exp_above3(sbx, sby, sbz);
       const sph::fx::Vec3 Sa = sph::vec64(sax, say, saz, esa), Sb = sph::vec64(sbx, sby, sbz, esb);
       const int kas = eca + esa - 2 * 1023 - 59, kbs = ecb + esb - 2 * 1023 - 59;
-      double dbx = sph::fx::scaled(sph::fx::dot(Ca[0], Sa), kas) +
-                   sph::fx::scaled(sph::fx::dot(Cb[0], Sb), kbs);
-      double dby = sph::fx::scaled(sph::fx::dot(Ca[1], Sa), kas) +
-                   sph::fx::scaled(sph::fx::dot(Cb[1], Sb), kbs);
-      double dbz = sph::fx::scaled(sph::fx::dot(Ca[2], Sa), kas) +
-                   sph::fx::scaled(sph::fx::dot(Cb[2], Sb), kbs);
+      double dbx = sph::fx::scaled<true>(sph::fx::dot(Ca[0], Sa), kas) +
+                   sph::fx::scaled<true>(sph::fx::dot(Cb[0], Sb), kbs);
+      double dby = sph::fx::scaled<true>(sph::fx::dot(Ca[1], Sa), kas) +
+                   sph::fx::scaled<true>(sph::fx::dot(Cb[1], Sb), kbs);
+      double dbz = sph::fx::scaled<true>(sph::fx::dot(Ca[2], Sa), kas) +
+                   sph::fx::scaled<true>(sph::fx::dot(Cb[2], Sb), kbs);
       // a value that is not finite has no fixed-point form: NaN instead
       if (max(max(ev, ecb == 0 ? 2048 : 0), max(esa, esb)) > 2047)
         dbx = __longlong_as_double(0x7ff8000000000000LL);
@@ -613,8 +632,28 @@ __global__ void __launch_bounds__(kThreads) k_adj_momentum_b(Slot sl, Work w, Pa
   }
 }
 
+// s = S d and d.S d in block fixed point: rows S times 2^(es - 1023), |d| below
+// 2^(ed - 1023).
+__device__ __forceinline__ double quadratic(const sph::fx::Vec3 S[3], int es, double dx, double dy,
+                                            double dz, int ed, double& s0, double& s1,
+                                            double& s2) {
+  const sph::fx::Vec3 D = sph::vec64(dx, dy, dz, ed);
+  const int k = es + ed - 2 * 1023 - 59;
+  const int64_t u0 = sph::fx::dot(S[0], D), u1 = sph::fx::dot(S[1], D), u2 = sph::fx::dot(S[2], D);
+  s0 = sph::fx::scaled<true>(u0, k);
+  s1 = sph::fx::scaled<true>(u1, k);
+  s2 = sph::fx::scaled<true>(u2, k);
+  sph::fx::Vec3 U;
+  sph::fx::put(U, 0, u0);
+  sph::fx::put(U, 1, u1);
+  sph::fx::put(U, 2, u2);
+  return sph::fx::scaled<true>(sph::fx::dot(U, D), k + ed - 1023 + 1);
+}
+
 // ---------------------------------------------------------------------------
-// Reverse of IAD's tau sums: tau_a = sum_b vol_b W_a d d^T, vol = m / rho.
+// Reverse of IAD's tau sums: tau_a = sum_b vol_b W_a d d^T, vol = m / rho.  The
+// FP64 pipe bounds it: S d and d.S d on the integer pipes leave 24 of 48 FP64
+// operations per pair (64,000 particles 0.79 -> 0.54 ms).
 // ---------------------------------------------------------------------------
 template <int NSUB>
 __global__ void __launch_bounds__(kThreads) k_adj_iad(Slot sl, Prep pr, Work w, PairBuf pb, Rev rv,
@@ -629,10 +668,13 @@ __global__ void __launch_bounds__(kThreads) k_adj_iad(Slot sl, Prep pr, Work w, 
   const bool valid = p_pair < n;
   const int64_t p = valid ? p_pair : n - 1;
   const double xp = s.x[p], yp = s.y[p], zp = s.z[p];
-  double Sp[6];
-#pragma unroll
-  for (int i = 0; i < 6; ++i) Sp[i] = w.Cb[6 * p + i];
-  double xbx = 0, xby = 0, xbz = 0;  // half of the adjoint of x_p
+  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  long long cf[6];
+  sph::fx::Vec3 S[3];
+  const int ep = sph::fix_matrix(w.Cb + 6 * p, cf);
+  sph::rows(cf, S);
+  const int ed = sph::fx::exp_above(2.0 * s.h[p]);  // |d| < 2 h_p
+  double xbx = ep == 0 ? nan : 0.0, xby = 0, xbz = 0;  // half of the adjoint of x_p
   // p's own sum: pairs (p, b)
   const int cnt = valid ? min(sl.nn[p], mb) : 0;
   const uint32_t* list = sl.nbr + p * mb;
@@ -643,8 +685,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_iad(Slot sl, Prep pr, Work w, 
     const double2 wk = pb.wk[(int64_t)k * pb.stride + p];
     const double vol = pr.vol[b];
     double s0, s1, s2;
-    sym_mv(Sp, dx, dy, dz, s0, s1, s2);
-    const double wbar = dx * s0 + dy * s1 + dz * s2;
+    const double wbar = quadratic(S, ep, dx, dy, dz, ed, s0, s1, s2);
     const double ww = vol * wk.x;
     const double f = wbar * (vol * wk.y);
     xbx -= ww * s0 + f * dx;
@@ -661,17 +702,15 @@ __global__ void __launch_bounds__(kThreads) k_adj_iad(Slot sl, Prep pr, Work w, 
     double dx = xp - s.x[a], dy = yp - s.y[a], dz = zp - s.z[a];
     sep64(im, dx, dy, dz);
     const double2 wk = pb.wk[k * pb.stride + a];
-    double Sa[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) Sa[i] = w.Cb[6 * a + i];
+    const int ea = sph::fix_matrix(w.Cb + 6 * a, cf);
+    sph::rows(cf, S);
     double s0, s1, s2;
-    sym_mv(Sa, dx, dy, dz, s0, s1, s2);
-    const double wbar = dx * s0 + dy * s1 + dz * s2;
+    const double wbar = quadratic(S, ea, dx, dy, dz, sph::exp_above3(dx, dy, dz), s0, s1, s2);
     const double f = wbar * wk.y;
     ybx += wk.x * s0 + f * dx;
     yby += wk.x * s1 + f * dy;
     ybz += wk.x * s2 + f * dz;
-    volbar += wbar * wk.x;
+    volbar += ea == 0 ? nan : wbar * wk.x;
   }
   const double volp = pr.vol[p];
   lanes_sum<NSUB>(fma(volp, ybx, xbx), sums[0]);
@@ -1064,7 +1103,7 @@ int build_rev(sph_adj* A, const Slot& sl, cudaStream_t st) {
   const int mb = A->prm.max_nb;
   cudaError_t e = cudaMemsetAsync(A->rcnt, 0, sizeof(int32_t) * (size_t)n, st);
   if (e != cudaSuccess) return acuda(A, e, "reverse lists");
-  const int g = grid_for(n, A->sm_count, 256, 16);
+  const int g = grid_for(n, A->sm_count, 256 / 32, 16);
   k_rev_count<<<g, 256, 0, st>>>(sl.nn, sl.nbr, mb, n, A->rcnt);
   sph::scan::exclusive_scan(A->rcnt, n, A->spart, A->rstart, st);
   e = cudaMemsetAsync(A->rcnt, 0, sizeof(int32_t) * (size_t)n, st);

@@ -219,13 +219,18 @@ SPH_FX int64_t dot(const Vec3& a, const Vec3& b) {
   return (hh << 2) + ((cr + (1 << 29)) >> 30);
 }
 
-// The double nearest to x 2^k; zero where that is below the normal range.
+// The double nearest to x 2^k; zero where that is below the normal range.  ANY:
+// infinity above it, for factors of any size (the forward pair sums, whose products
+// stay inside, would spend 2% on the compare).
+template <bool ANY = false>
 SPH_FX double scaled(int64_t x, int k) {
   const int64_t g = x >> 63;
   const uint64_t u = (uint64_t)((x ^ g) - g);
   const int z = clz64(u);
   const int f = 1085 + k - z;  // exponent field, less the implicit bit
-  if (u == 0 || f < 0) return 0.0;
+  if (u == 0 || (ANY ? (uint32_t)f > 2045u : f < 0))
+    return ANY && u != 0 && f > 0
+               ? from_bits((uint64_t)0x7ff0000000000000 | ((uint64_t)g << 63)) : 0.0;
   const uint64_t m = u << z;
   return from_bits((((uint64_t)(uint32_t)f << 52) + (m >> 11) + ((m >> 10) & 1u)) |
                    ((uint64_t)g << 63));

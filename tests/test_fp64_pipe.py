@@ -42,6 +42,7 @@ extern "C" void dots(const double* a, const double* b, double* out, long n) {
     out[i] = scaled(dot(A, B), ea + eb - 2 * 1023 - 59);
   }
 }
+extern "C" double edge(long x, int k) { return sph::fx::scaled<true>(x, k); }
 // for d (3 per entry), 2 h_a, 1 / h_b^2, v, a: S^6 at t = r^2 / h_b^2, its product with a, v.d / r
 // (0 where r is below 1/16 of the power of two above 2 h_a), and (a S^6) d_x
 extern "C" void pair(const double* d, const double* h2, const double* hinv2, const double* v,
@@ -92,6 +93,7 @@ def fixed(tmp_path_factory):
         out = [np.empty_like(t) for _ in range(3)]
         f.eval(*[a.ctypes.data_as(C.c_void_p) for a in (t, *out)], C.c_long(t.size))
         return out
+    run.edge = f.edge
     return run
 
 
@@ -277,3 +279,45 @@ def test_fp64_close_pairs_and_uneven_h(opts):
     e = field_errors(got, ref)
     for k in ("rho", "p", "c", "iad", "a", "du"):
         assert e[k] <= 1e-12, (k, e)
+
+
+def test_scaled_past_the_range(fixed):
+    fixed.edge.restype = C.c_double
+    fixed.edge.argtypes = [C.c_long, C.c_int]
+    for x in (1, -1, 3, (1 << 62) - 1, -(1 << 61)):
+        for k in (-1200, -1023, -80, 0, 900, 962, 1023, 1100, 3000):
+            want = np.ldexp(float(x), k) if abs(np.ldexp(float(x), k)) >= 2.0 ** -1022 else 0.0
+            assert fixed.edge(x, k) == want, (x, k)
+    assert fixed.edge(0, 3000) == 0.0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("side,ng", [(8, 20), (12, 150), (16, 620)])
+def test_reverse_lists_of_every_length(side, ng):
+    """Reverse lists below, at and past the 128 entries a warp ranks at a time and the 512 it
+    keeps in shared memory, by the closed forms of a rollout's gradient: sum_a dL/dx_a = 0 and
+    sum_a dL/dv_a = sum_a m_a v_a(K) within the FP64 bound on sums of n terms (1e-10 of the
+    terms' sum of magnitudes); and the same bits from a second reverse pass."""
+    import torch
+
+    from paper_2005_02656_gb300 import Params, Rollout
+    s = sph_inputs.jittered_box(side, seed_index=91, vel_sigma=0.05)
+    s["h"][:] = 0.5 / side * (3.0 * ng / (4.0 * np.pi)) ** (1.0 / 3.0)
+    ro = Rollout(side ** 3, 2, 1, Params(box_lo=s["lo"], box_hi=s["hi"], periodic=s["periodic"],
+                                         max_nb=1024, ng_target=0))
+    st = {k: torch.as_tensor(s[k], dtype=torch.float64, device=ro.device)
+          for k in ("x", "y", "z", "vx", "vy", "vz", "vxh", "vyh", "vzh", "h", "m", "u", "du_prev")}
+    fin = ro.forward(st, 1.0)
+    g = torch.zeros_like(fin)
+    g[3:6] = st["m"][None, :] * fin[3:6]
+    g[7] = 2.0 * (fin[7] - 1.0)
+    gi, ga = ro.backward(g)
+    again, _ = ro.backward(g)
+    assert torch.equal(gi, again)
+    ro.close()
+    gi = gi.cpu().numpy()
+    p = (s["m"][None, :] * fin[3:6].cpu().numpy())
+    for k in range(3):
+        assert abs(gi[k].sum()) <= 1e-10 * np.abs(gi[k]).sum()
+        dv = gi[3 + k] + gi[6 + k]
+        assert abs(dv.sum() - p[k].sum()) <= 1e-10 * (np.abs(dv).sum() + np.abs(p[k]).sum())
