@@ -23,6 +23,9 @@
 //      are bit-identical to r^2 < (2h)^2 evaluated in FP64 without FMA;
 //   3. each lane appends its hits of the block, in slot order, from a 64-bit
 //      hit mask.
+// Where the particles are too few for the chip (SHARE) several warps share the
+// targets of a cell, in rounds of 8, four lanes to a target: each lane takes its
+// own block of 64, and its appends start after the hits of the lower blocks.
 // Lists are uint32 entries (particle index + cell-shift code, sph_tile.cuh),
 // row-major per particle: nbr[a * max_nb + k], in stencil-slot order.
 #pragma once
@@ -58,14 +61,17 @@ __device__ __forceinline__ int pair_index(int i) {
   return (blk << 6) + ((r & 31) << 1) + (r >> 5);
 }
 
-template <int WIN>
+// PAD: floats between blocks (2: lanes that read the same pair of different
+// blocks meet no bank twice).
+template <int WIN, int PAD = 0>
 struct FindWarpSmemT {
   static_assert(WIN % 64 == 0, "the window holds whole blocks of 64 slots");
   Stencil S;
   // 16-byte aligned: the candidate arrays are read as float2 pairs
-  alignas(16) float cx[WIN];
-  alignas(16) float cy[WIN];
-  alignas(16) float cz[WIN];
+  static constexpr int kFloats = ((64 + PAD) * (WIN / 64) + 3) / 4 * 4;
+  alignas(16) float cx[kFloats];
+  alignas(16) float cy[kFloats];
+  alignas(16) float cz[kFloats];
   uint32_t entry[WIN];  // list entry of each staged slot (sph_tile.cuh)
 };
 using FindWarpSmem = FindWarpSmemT<kFindWindow>;
@@ -115,15 +121,18 @@ __device__ __forceinline__ void block_masks(const Grid& g, const float* cx, cons
 constexpr uint64_t kTop = 1ull << 63;
 
 // Builds the lists of every target of occupied cell `code` (one warp; the
-// warp owns W, a window of WIN staged slots).  Counts tested candidates and
-// exact FP64 tests.
-template <bool WRAP, int WIN = kFindWindow>
+// warp owns W, a window of WIN staged slots; SHARE: of `parts` warps that call it
+// for a cell, warp `part` takes every parts-th round of targets).  Counts tested
+// candidates and exact FP64 tests.
+template <bool WRAP, int WIN = kFindWindow, bool SHARE = false>
 __device__ __forceinline__ void find_cell(const Grid& g, uint32_t code, const StateView& s,
                                           const float4* __restrict__ pos32,
                                           const uint32_t* tbl_start, const uint32_t* tbl_count,
                                           int32_t* nn, uint32_t* nbr, int max_nb, uint32_t* err,
-                                          FindWarpSmemT<WIN>& W, unsigned long long& tested,
-                                          unsigned long long& exact) {
+                                          FindWarpSmemT<WIN, SHARE ? 2 : 0>& W,
+                                          unsigned long long& tested,
+                                          unsigned long long& exact, int part = 0,
+                                          int parts = 1) {
   const int lane = threadIdx.x & 31;
   Stencil& S = W.S;
   const float esum = g.err32[0] + g.err32[1] + g.err32[2];
@@ -171,6 +180,11 @@ __device__ __forceinline__ void find_cell(const Grid& g, uint32_t code, const St
     __syncwarp();
   }
 
+  constexpr int kBlock = SHARE ? 66 : 64;      // floats per block of 64 slots
+  constexpr int kLanes = SHARE ? 4 : 1;        // lanes per target
+  constexpr int kRound = 32 / kLanes;          // targets per round
+  const int own64 = 64 * (lane / kRound);      // first slot of the lane's block
+
   int wn = 0;           // slots staged in the current window
   int wbase = 0;        // staged slots before the current window
   int gself = -1;       // staged index of the target cell's first particle
@@ -213,7 +227,7 @@ __device__ __forceinline__ void find_cell(const Grid& g, uint32_t code, const St
         const uint32_t bal = __ballot_sync(0xffffffffu, keep);
         if (keep) {
           const int q = wn + __popc(bal & lt);
-          const int pq = pair_index(q);
+          const int pq = pair_index(q) + (kBlock - 64) * (q >> 6);
           W.cx[pq] = cx;
           W.cy[pq] = cy;
           W.cz[pq] = cz;
@@ -230,14 +244,14 @@ __device__ __forceinline__ void find_cell(const Grid& g, uint32_t code, const St
     // the targets of the cell against the staged window
     const int wpad = (wn + 63) & ~63;
     for (int i = wn + lane; i < wpad; i += 32) {
-      const int q = pair_index(i);
+      const int q = pair_index(i) + (kBlock - 64) * (i >> 6);
       W.cx[q] = kFar;
       W.cy[q] = kFar;
       W.cz[q] = kFar;
     }
     __syncwarp();
-    for (int t0 = 0; t0 < na; t0 += 32) {
-      const int t = t0 + lane;
+    for (int t0 = part * kRound; t0 < na; t0 += parts * kRound) {
+      const int t = t0 + lane % kRound;
       const bool active = t < na;
       const int a = a0 + (active ? t : 0);
       const float4 pa = pos32[a];
@@ -250,10 +264,15 @@ __device__ __forceinline__ void find_cell(const Grid& g, uint32_t code, const St
       const int gs = gself >= 0 ? gself + t - wbase : -1;
       const int self = (active && gs >= 0 && gs < wn) ? gs : -1;
       int k = (first || !active) ? 0 : nn[a];
-      for (int jb = 0; jb < wpad; jb += 64) {
+      for (int jw = 0; jw < wpad; jw += 64 * kLanes) {
+        // the lane's block; past the last block, the first one again for nothing
+        const bool has = !SHARE || jw + own64 < wpad;
+        const int jb = has ? jw + own64 : jw;
+        const int cb = (jb >> 6) * kBlock;
         uint64_t hit, unc;
-        block_masks<WRAP>(g, W.cx + jb, W.cy + jb, W.cz + jb, npx, npy, npz, lo_lim, hi_lim,
+        block_masks<WRAP>(g, W.cx + cb, W.cy + cb, W.cz + cb, npx, npy, npz, lo_lim, hi_lim,
                           hit, unc);
+        if (SHARE && !has) hit = unc = 0;
         // candidates inside the margin: exact FP64 test
         while (unc) {
           const int q = __clzll((long long)unc);
@@ -265,19 +284,31 @@ __device__ __forceinline__ void find_cell(const Grid& g, uint32_t code, const St
         }
         if (self >= jb && self < jb + 64) hit &= ~(kTop >> (self - jb));
         if (!active) hit = 0;
+        int at = k;
+        if (SHARE) {  // the hits of the target's lower blocks come first
+          int c = __popcll(hit);
+          const int c1 = __shfl_xor_sync(0xffffffffu, c, kRound);
+          if (lane & kRound) at += c1;
+          c += c1;
+          const int c2 = __shfl_xor_sync(0xffffffffu, c, 2 * kRound);
+          if (lane & (2 * kRound)) at += c2;
+          k += c + c2;
+        }
         uint32_t* row = nbr + (int64_t)a * max_nb;
         while (hit) {  // slot order
           const int q = __clzll((long long)hit);
           hit ^= kTop >> q;
-          if (k < max_nb) row[k] = W.entry[jb + q];
-          ++k;
+          if (at < max_nb) row[at] = W.entry[jb + q];
+          ++at;
         }
+        if (!SHARE) k = at;
       }
-      if (active) {
+      if (active && own64 == 0) {
         nn[a] = k;
         if (k > max_nb) raise_flag(err, SPH_FLAG_NB_OVERFLOW);
         tested += (unsigned long long)wn - (self >= 0 ? 1 : 0);
       }
+      if (SHARE) __syncwarp();
     }
     __syncwarp();
     first = false;

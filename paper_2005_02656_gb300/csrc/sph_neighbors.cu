@@ -18,28 +18,42 @@ namespace {
 
 using namespace find;
 
+// SHARE: up to this many particles per SM several warps share a cell (a warp per
+// cell leaves most of the chip idle and takes its rounds one after the other):
+// 4,096 particles 61 -> 33 us, 8,000 64 -> 35, 13,824 35 -> 29, 21,952 62 -> 43;
+// 32,768 are as fast or faster with a warp per cell (40 us; two rounds a cell need
+// more than 32 particles in it).
+constexpr int64_t kShareN = 160;
+
 // No register cap: at 108-122 registers (4 CTAs per SM) the search measured
 // 1-2% faster than capped at 94 (5 CTAs) or 80 (6 CTAs); its unrolled mask
-// loop gains more from registers than from resident warps.
-__global__ void __launch_bounds__(kFindThreads, 1) k_find_tile(
+// loop gains more from registers than from resident warps.  SHARE holds four CTAs.
+template <bool SHARE>
+__global__ void __launch_bounds__(kFindThreads, SHARE ? 4 : 1) k_find_tile(
     const Grid* gp, StateView s, const float4* __restrict__ pos32, const uint32_t* occ,
     const uint32_t* tbl_start, const uint32_t* tbl_count, int32_t* nn, uint32_t* nbr,
     int max_nb, uint32_t* err, unsigned long long* stats) {
   dep_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  FindWarpSmem& W = reinterpret_cast<FindWarpSmem*>(smem_raw)[warp];
+  using Smem = FindWarpSmemT<kFindWindow, SHARE ? 2 : 0>;
+  Smem& W = reinterpret_cast<Smem*>(smem_raw)[warp];
   const Grid g = *gp;
   unsigned long long tested = 0, exact = 0;
   const uint32_t gw = blockIdx.x * kFindWarps + warp, nw = gridDim.x * kFindWarps;
+  // warps per cell: what the grid holds over the occupied cells, 8 at most
+  const uint32_t parts = SHARE ? min(max(nw / max(g.n_occ, 1u), 1u), 8u) : 1u;
+  const uint32_t items = g.n_occ * parts;
   if (g.wrap32) {  // a periodic axis with fewer than 3 cells: FP32 separations need the wrap
-    for (uint32_t cell = gw; cell < g.n_occ; cell += nw)
-      find_cell<true>(g, occ[cell], s, pos32, tbl_start, tbl_count, nn, nbr, max_nb, err, W,
-                      tested, exact);
+    for (uint32_t it = gw; it < items; it += nw)
+      find_cell<true, kFindWindow, SHARE>(g, occ[it / parts], s, pos32, tbl_start, tbl_count, nn,
+                                          nbr, max_nb, err, W, tested, exact, (int)(it % parts),
+                                          (int)parts);
   } else {
-    for (uint32_t cell = gw; cell < g.n_occ; cell += nw)
-      find_cell<false>(g, occ[cell], s, pos32, tbl_start, tbl_count, nn, nbr, max_nb, err, W,
-                       tested, exact);
+    for (uint32_t it = gw; it < items; it += nw)
+      find_cell<false, kFindWindow, SHARE>(g, occ[it / parts], s, pos32, tbl_start, tbl_count, nn,
+                                           nbr, max_nb, err, W, tested, exact, (int)(it % parts),
+                                           (int)parts);
   }
   // counters: one atomic per warp
   for (int o = 16; o > 0; o >>= 1) {
@@ -76,18 +90,23 @@ __global__ void k_export(int64_t n, const int32_t* nn, const uint32_t* nbr, int 
 }  // namespace
 
 void launch_find_neighbors(sph_ctx* ctx, const StateView& s, int64_t n, cudaStream_t st) {
-  (void)n;
-  const size_t smem = kFindWarps * sizeof(FindWarpSmem);
+  const bool share = n <= kShareN * ctx->sm_count;
+  const size_t smem = kFindWarps * (share ? sizeof(FindWarpSmemT<kFindWindow, 2>)
+                                          : sizeof(FindWarpSmem));
   if (!ctx->find_blocks) {  // once per context, on its device
     int per_sm = 0;
-    cudaFuncSetAttribute(k_find_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_find_tile, kFindThreads,
-                                                  smem);
+    cudaFuncSetAttribute(k_find_tile<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(kFindWarps * sizeof(FindWarpSmem)));
+    cudaFuncSetAttribute(k_find_tile<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(kFindWarps * sizeof(FindWarpSmemT<kFindWindow, 2>)));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_find_tile<false>, kFindThreads,
+                                                  kFindWarps * sizeof(FindWarpSmem));
     ctx->find_blocks = (per_sm > 0 ? per_sm : 1) * ctx->sm_count;
   }
-  launch_dep(k_find_tile, ctx->find_blocks, kFindThreads, smem, st, ctx->grid, s, ctx->pos32,
-             ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb, ctx->err,
-             ctx->stats);
+  launch_dep(share ? k_find_tile<true> : k_find_tile<false>,
+             share ? 4 * ctx->sm_count : ctx->find_blocks, kFindThreads, smem, st, ctx->grid, s,
+             ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr,
+             ctx->prm.max_nb, ctx->err, ctx->stats);
   ctx->launches += 1;
 }
 
