@@ -18,8 +18,8 @@
 //  - scalar products are block fixed point, and with S^6 (FAST) so are r^2, v
 //    and 1/r, from the separation's fixed-point form;
 //  - the per-target work runs on whole warps (lanes_sum).
-// Per pair about 4 (density), 9 (IAD) and 28 (momentum) FP64 operations; at
-// 1.07M particles 1.82, 2.86 and 7.99 ms, where the FP64 series, products and
+// Per pair about 4 (density), 9 (IAD) and 26 (momentum) FP64 operations; at
+// 1.07M particles 1.82, 2.86 and 7.66 ms (7.99 with C_a applied to every pair), where the FP64 series, products and
 // comparisons with one thread per target took 7.38, 4.11 and 20.6 ms.
 #include <cuda_runtime.h>
 #include "sph_device.cuh"
@@ -299,15 +299,17 @@ __global__ void __launch_bounds__(kThreads64, 4) k_momentum64(const Grid* gp, co
   const Rec64* ra = rec + a;
   const double xa = ra->x, ya = ra->y, za = ra->z;
   const double vxa = ra->vx, vya = ra->vy, vza = ra->vz;
-  const double Xa = ra->X, ira = ra->irq, ca = ra->c;
+  const double Xa = ra->X, ira = ra->irq, hira = 0.5 * ira, ca = ra->c;
   const int ed = fx::exp_above(2.0 * s.h[a]);  // |d| < 2 h_a
   fx::Vec3 Ca[3];
   rows(ra->cf, Ca);
   const int cnt = valid ? min(L.nn[a], L.max_nb) : 0;
   const uint32_t* list = L.nbr + a * L.max_nb;
   const double* wrow = L.w + a * L.max_nb;
-  double accx = 0, accy = 0, accz = 0, du = 0;      // terms of W_a, without B_n/h_a^3
+  // sum fa d and the terms of W_a, without B_n/h_a^3 (C_a is applied to the sum)
+  double accx = 0, accy = 0, accz = 0, du = 0;
   double bccx = 0, bccy = 0, bccz = 0, dub = 0;     // terms of W_b
+  bool bad = false;                                 // a velocity that is not finite
   for (int k = sub; k < cnt; k += NSUB) {
     const Rec64* rb = rec + entry_index(list[k]);
     double dx = rb->x - xa, dy = rb->y - ya, dz = rb->z - za;
@@ -316,7 +318,7 @@ __global__ void __launch_bounds__(kThreads64, 4) k_momentum64(const Grid* gp, co
     const fx::Vec3 D = vec64(dx, dy, dz, ed);
     const int ev = exp_above3(vx, vy, vz);
     const fx::Vec3 V = vec64(vx, vy, vz, ev);
-    const double vnan = ev <= 2047 ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
+    bad |= ev > 2047;
     const int64_t vd = fx::dot(V, D);  // -x_ab . v_ab
     const int kv = ev + ed - 2 * 1023 - 60, kr = 2 * (ed - 1023) - 60;
     const int64_t R = FAST ? fx::dot(D, D) : 0;
@@ -336,27 +338,22 @@ __global__ void __launch_bounds__(kThreads64, 4) k_momentum64(const Grid* gp, co
         wv = fma(z, e, z);
       }
     }
-    double pa = 0.0, pb = 0.0;
+    double q = 0.0, pb = 0.0;
     if (vd > 0) {
-      const double q = wv * fma(3.0, wv, -(ca + rb->c));
-      pa = q * ira;
+      q = wv * fma(3.0, wv, -(ca + rb->c));
       pb = q * rb->irq;
     }
     const double wa = rb->m * wrow[k];
-    const double fa = wa * (Xa + pa);
+    const double fa = wa * fma(q, ira, Xa);
     const double fb = wb * (rb->X + pb);
+    accx += fa * dx;
+    accy += fa * dy;
+    accz += fa * dz;
     {
-      int64_t U[3];
       fx::Vec3 Uv;
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        U[i] = fx::dot(Ca[i], D);
-        fx::put(Uv, i, U[i]);
-      }
-      accx += fa * fx::scaled(U[0], 0);
-      accy += fa * fx::scaled(U[1], 0);
-      accz += fa * fx::scaled(U[2], 0);
-      du += wa * fma(0.5, pa, Xa) * (fx::scaled(fx::dot(V, Uv), ev - 1023) + vnan);
+      for (int i = 0; i < 3; ++i) fx::put(Uv, i, fx::dot(Ca[i], D));
+      du += wa * fma(q, hira, Xa) * fx::scaled(fx::dot(V, Uv), ev - 1023);
     }
     {
       fx::Vec3 Cb[3], Uv;
@@ -377,11 +374,13 @@ __global__ void __launch_bounds__(kThreads64, 4) k_momentum64(const Grid* gp, co
   // v.C d = R 2^(e_v + e_C + e_d - 58)
   long long cf[6];
   const double pd = power_of(ed) * 0x1p-59;
-  const double pn = aux.wnorm[a] * power_of(fix_matrix(o.iad + 6 * a, cf)) * pd;
-  lanes_sum<NSUB>(fma(-pn, accx, -pd * bccx), sums[0]);
-  lanes_sum<NSUB>(fma(-pn, accy, -pd * bccy), sums[1]);
-  lanes_sum<NSUB>(fma(-pn, accz, -pd * bccz), sums[2]);
-  lanes_sum<NSUB>(2.0 * fma(pn, du, 0.5 * pd * dub), sums[3]);
+  const double* C = o.iad + 6 * a;
+  const double wn = aux.wnorm[a], pn = wn * power_of(fix_matrix(C, cf)) * pd;
+  lanes_sum<NSUB>(fma(-wn, C[0] * accx + C[1] * accy + C[2] * accz, -pd * bccx), sums[0]);
+  lanes_sum<NSUB>(fma(-wn, C[1] * accx + C[3] * accy + C[4] * accz, -pd * bccy), sums[1]);
+  lanes_sum<NSUB>(fma(-wn, C[2] * accx + C[4] * accy + C[5] * accz, -pd * bccz), sums[2]);
+  du = 2.0 * fma(pn, du, 0.5 * pd * dub);
+  lanes_sum<NSUB>(bad ? __longlong_as_double(0x7ff8000000000000LL) : du, sums[3]);
   __syncthreads();
   a = blockIdx.x * (int64_t)kT + threadIdx.x;
   if (threadIdx.x >= kT || a >= n) return;
