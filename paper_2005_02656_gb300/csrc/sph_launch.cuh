@@ -13,12 +13,22 @@
 
 namespace sph {
 
+// The searches are persistent and take most of an SM's shared memory: launched
+// early, some of their CTAs meet an SM that still runs the gather with a small
+// shared-memory share, start late, and the whole share of cells they own with them.
+// Early against plain (us per step): staged search 8,000 particles 135.5 / 139.2,
+// 103,823 (stage calls) 307.4 / 311.2, 125,000: 405.8 / 400.5, 250,047: 607.8 /
+// 612.3, 512,000: 1,141 / 1,125, 8.4M: 14,864 / 14,630; list search (FP64) 8,000:
+// 246.3 / 247.7, 32,768: 617 / 601, 250,047: 3,379 / 3,364, 1.07M: 13,735 / 13,660.
+constexpr int64_t kEarlyMasksN = 400000;
+constexpr int64_t kEarlyListsN = 20000;
+
 template <class... P, class... A>
-inline void launch_dep(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
-                       cudaStream_t st, A&&... args) {
+inline void launch_dep_if(bool early, void (*kernel)(P...), unsigned grid, unsigned block,
+                          size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
+  at.val.programmaticStreamSerializationAllowed = early ? 1 : 0;
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3(grid);
   c.blockDim = dim3(block);
@@ -27,6 +37,12 @@ inline void launch_dep(void (*kernel)(P...), unsigned grid, unsigned block, size
   c.attrs = &at;
   c.numAttrs = 1;
   cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
+template <class... P, class... A>
+inline void launch_dep(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                       cudaStream_t st, A&&... args) {
+  launch_dep_if(true, kernel, grid, block, smem, st, std::forward<A>(args)...);
 }
 
 // Waits for the kernels before this one in the stream, then lets the next

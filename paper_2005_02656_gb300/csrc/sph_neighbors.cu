@@ -103,7 +103,7 @@ void launch_find_neighbors(sph_ctx* ctx, const StateView& s, int64_t n, cudaStre
                                                   kFindWarps * sizeof(FindWarpSmem));
     ctx->find_blocks = (per_sm > 0 ? per_sm : 1) * ctx->sm_count;
   }
-  launch_dep(share ? k_find_tile<true> : k_find_tile<false>,
+  launch_dep_if(n < kEarlyListsN, share ? k_find_tile<true> : k_find_tile<false>,
              share ? 4 * ctx->sm_count : ctx->find_blocks, kFindThreads, smem, st, ctx->grid, s,
              ctx->pos32, ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr,
              ctx->prm.max_nb, ctx->err, ctx->stats);

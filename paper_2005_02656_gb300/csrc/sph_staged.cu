@@ -1867,7 +1867,7 @@ void launch_find_masks(sph_ctx* ctx, const StateView& s, int64_t n, cudaStream_t
   // 43, 8,000: 57 / 42, 13,824: 36 / 38, 21,952: 57 / 65).
   const int64_t cta_max = 64 * (int64_t)ctx->sm_count;
   auto run = [&](auto kernel) {
-    launch_dep(kernel, ctx->find_mask_blocks, kFindThreads, smem, st, ctx->grid, s, ctx->pos32,
+    launch_dep_if(n < kEarlyMasksN, kernel, ctx->find_mask_blocks, kFindThreads, smem, st, ctx->grid, s, ctx->pos32,
                ctx->occ, ctx->tbl_start, ctx->tbl_count, ctx->nn, ctx->nbr, ctx->prm.max_nb, mo,
                ctx->err, ctx->stats);
   };
