@@ -33,11 +33,12 @@ SAMPLE_NX = 112        # the same recipe at 1/8 scale for the CPU oracle (1,067,
 
 # Flop model per directed neighbour pair (add/sub/mul = 1, FMA = 2,
 # rsqrt/div = 1), counted on the operations of each pair loop as written; the
-# neighbour search counts per (target, candidate) test.  The FP64 kernels
-# evaluate a 15-term series for W (32 flops, 7 terms in FP32) and IAD and
-# momentum read W_ab(h_a) cached by the density pass.
+# neighbour search counts per (target, candidate) test.  IAD and
+# momentum of the FP64 path read S^6 cached by the density pass.
 FLOPS = {"find": 14, "density": 37, "iad": 57, "momentum": 140}
-FLOPS64 = {"find": 14, "density": 43, "iad": 19, "momentum": 131}
+# of the 43 / 19 / 131 FP64 operations of the formulas, those the FP64 pipe executes
+# (the kernel series, roots and scalar products run in fixed point on the integer pipes)
+FLOPS64 = {"find": 14, "density": 6, "iad": 16, "momentum": 38}
 # Algorithmic HBM bytes of each kernel launch, every array it touches read or
 # written once: per particle (its own fields in and out; the records of
 # neighbours counted once, as the particle's own record), per staged slot (the
