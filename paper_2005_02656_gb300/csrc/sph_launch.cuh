@@ -22,6 +22,11 @@ namespace sph {
 // 246.3 / 247.7, 32,768: 617 / 601, 250,047: 3,379 / 3,364, 1.07M: 13,735 / 13,660.
 constexpr int64_t kEarlyMasksN = 400000;
 constexpr int64_t kEarlyListsN = 20000;
+// The FP64 pair kernels: early CTAs take slots from the end of the pass before
+// them.  Early against plain (us): 32,768 particles 601 / 606, 64,000 (20 steps and
+// gradient, ms) 109.9 / 110.1, 125,000: 1,845 / 1,837, 1.07M: 13,700 / 13,521,
+// 1.0M square patch (stage calls) 10,658 / 10,511.
+constexpr int64_t kEarlyPairsN = 100000;
 
 template <class... P, class... A>
 inline void launch_dep_if(bool early, void (*kernel)(P...), unsigned grid, unsigned block,
