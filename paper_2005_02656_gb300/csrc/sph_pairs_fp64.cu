@@ -436,9 +436,9 @@ void launch_density_f64(sph_ctx* ctx, const StateView& s, const OutView& o, int6
     auto kern = ctx->prm.gradh ? k_density64<NS, true, false>
                                : (fast64(ctx) ? k_density64<NS, false, true>
                                               : k_density64<NS, false, false>);
-    launch_dep_if(n < kEarlyPairsN, kern, blocks64(n, NS), kThreads64, 0, st, ctx->grid, s, o, aux_of(ctx),
-        lists64_of(ctx), n, ctx->Bn, (int)ctx->prm.sinc_n, ctx->prm.gamma, ctx->prm.alpha,
-        ctx->err);
+    launch_dep_if(n < kEarlyPairsN, kern, blocks64(n, NS), kThreads64, 0, st, ctx->grid, s, o,
+                  aux_of(ctx), lists64_of(ctx), n, ctx->Bn, (int)ctx->prm.sinc_n, ctx->prm.gamma,
+                  ctx->prm.alpha, ctx->err);
   });
   ctx->launches += 1;
 }
@@ -447,8 +447,8 @@ void launch_iad_f64(sph_ctx* ctx, const StateView& s, const OutView& o, int64_t 
                     cudaStream_t st) {
   with_lanes64(n, [&](auto lanes) {
     constexpr int NS = decltype(lanes)::value;
-    launch_dep_if(n < kEarlyPairsN, k_iad64<NS>, blocks64(n, NS), kThreads64, 0, st, ctx->grid, s, o, aux_of(ctx),
-        lists64_of(ctx), n, ctx->err);
+    launch_dep_if(n < kEarlyPairsN, k_iad64<NS>, blocks64(n, NS), kThreads64, 0, st, ctx->grid, s,
+                  o, aux_of(ctx), lists64_of(ctx), n, ctx->err);
   });
   ctx->launches += 1;
 }
@@ -459,12 +459,13 @@ void launch_momentum_f64(sph_ctx* ctx, const StateView& s, const OutView& o, int
   // (a search of either form writes its own before it is read)
   static_assert(sizeof(Rec64) <= kMaskWords * sizeof(unsigned long long), "fits the mask buffer");
   Rec64* rec = reinterpret_cast<Rec64*>(ctx->masks);
-  launch_dep_if(n < kEarlyPairsN, k_pack64, (unsigned)((n + 127) / 128), 128, 0, st, s, o, aux_of(ctx), n, rec);
+  launch_dep_if(n < kEarlyPairsN, k_pack64, (unsigned)((n + 127) / 128), 128, 0, st, s, o,
+                aux_of(ctx), n, rec);
   with_lanes64(n, [&](auto lanes) {
     constexpr int NS = decltype(lanes)::value;
     auto kern = fast64(ctx) ? k_momentum64<NS, true> : k_momentum64<NS, false>;
     launch_dep_if(n < kEarlyPairsN, kern, blocks64(n, NS), kThreads64, 0, st, ctx->grid, rec, s, o,
-        aux_of(ctx), lists64_of(ctx), n, (int)ctx->prm.sinc_n, ctx->err);
+                  aux_of(ctx), lists64_of(ctx), n, (int)ctx->prm.sinc_n, ctx->err);
   });
   ctx->launches += 2;
 }
