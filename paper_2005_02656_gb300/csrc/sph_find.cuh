@@ -126,7 +126,7 @@ constexpr uint64_t kTop = 1ull << 63;
 // candidates and exact FP64 tests.
 template <bool WRAP, int WIN = kFindWindow, bool SHARE = false>
 __device__ __forceinline__ void find_cell(const Grid& g, uint32_t code, const StateView& s,
-                                          const float4* __restrict__ pos32,
+                                          const float4* pos32,
                                           const uint32_t* tbl_start, const uint32_t* tbl_count,
                                           int32_t* nn, uint32_t* nbr, int max_nb, uint32_t* err,
                                           FindWarpSmemT<WIN, SHARE ? 2 : 0>& W,

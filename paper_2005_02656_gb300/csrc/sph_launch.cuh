@@ -4,7 +4,12 @@
 // visible.  The launch latency and the block start-up of each kernel then hide
 // behind its predecessor, which is a large part of a small state's step (about
 // 30 launches).  Every kernel launched this way calls dep_enter before it
-// touches memory.
+// touches memory.  What the kernel before it in the stream writes is read by
+// ordinary loads only: the read-only path (__ldg, const __restrict__ parameters)
+// is for data that nobody writes while the grid exists, and dep_enter does not
+// order it.  What was written two or more kernels back is complete when a
+// kernel's blocks are scheduled (the one between was past its wait), and may be
+// read either way.
 #pragma once
 
 #include <cuda_runtime.h>

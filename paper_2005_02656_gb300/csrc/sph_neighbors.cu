@@ -30,7 +30,7 @@ constexpr int64_t kShareN = 160;
 // loop gains more from registers than from resident warps.  SHARE holds four CTAs.
 template <bool SHARE>
 __global__ void __launch_bounds__(kFindThreads, SHARE ? 4 : 1) k_find_tile(
-    const Grid* gp, StateView s, const float4* __restrict__ pos32, const uint32_t* occ,
+    const Grid* gp, StateView s, const float4* pos32, const uint32_t* occ,
     const uint32_t* tbl_start, const uint32_t* tbl_count, int32_t* nn, uint32_t* nbr,
     int max_nb, uint32_t* err, unsigned long long* stats) {
   dep_enter();

@@ -156,7 +156,7 @@ struct PartShared {
 template <bool WRAP, int WIN, int PARTS>
 __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, uint32_t code,
                                                 const StateView& s,
-                                                const float4* __restrict__ pos32,
+                                                const float4* pos32,
                                                 const uint32_t* tbl_start,
                                                 const uint32_t* tbl_count, int32_t* nn,
                                                 uint32_t* nbr, int max_nb, const MaskOut& mo,
@@ -449,7 +449,7 @@ __device__ __forceinline__ void find_cell_masks(const Grid& g, uint32_t cell, ui
 // Capped at 128 registers so that four CTAs stay resident per SM.
 template <bool WRAP>
 __global__ void __launch_bounds__(kFindThreads, 4) k_find_mask(
-    const Grid* gp, StateView s, const float4* __restrict__ pos32, const uint32_t* occ,
+    const Grid* gp, StateView s, const float4* pos32, const uint32_t* occ,
     const uint32_t* tbl_start, const uint32_t* tbl_count, int32_t* nn, uint32_t* nbr, int max_nb,
     MaskOut mo, uint32_t* err, unsigned long long* stats) {
   dep_enter();
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kFindThreads, 4) k_find_mask(
 // warp one (launch_find_masks).
 template <bool WRAP>
 __global__ void __launch_bounds__(kFindThreads, 4) k_find_mask_cta(
-    const Grid* gp, StateView s, const float4* __restrict__ pos32, const uint32_t* occ,
+    const Grid* gp, StateView s, const float4* pos32, const uint32_t* occ,
     const uint32_t* tbl_start, const uint32_t* tbl_count, int32_t* nn, uint32_t* nbr, int max_nb,
     MaskOut mo, uint32_t* err, unsigned long long* stats) {
   dep_enter();
@@ -1183,12 +1183,12 @@ __device__ __forceinline__ void prefetch_cell(const Src& src, uint4 md,
   const int tid = threadIdx.x;
   const int S = cell_S(md), na = cell_na(md);
   const bool staged = md.y != kListForm;
-  pf.nn = (staged && tid < kTR && tid < na) ? __ldg(src.nn + md.z + tid) : 0;
+  pf.nn = (staged && tid < kTR && tid < na) ? src.nn[md.z + tid] : 0;
   const int wn = min(Pass::kWin, S);
 #pragma unroll
   for (int i = 0; i < window_slots<Pass>(); ++i) {
     const int j = tid + i * kPT;
-    pf.e[i] = (staged && j < wn) ? __ldg(src.sent + md.x + (uint32_t)j) : 0u;
+    pf.e[i] = (staged && j < wn) ? src.sent[md.x + (uint32_t)j] : 0u;
   }
 }
 
@@ -1210,9 +1210,9 @@ __device__ __forceinline__ void cellpass(const Pass& pass, const Grid* gp, const
   tb.fill<kPT>(g);
   const int tid = threadIdx.x;
   const uint4 zero4 = make_uint4(0u, kListForm, 0u, 0u);
-  auto meta_of = [&](uint32_t q) { return q < n_cells ? __ldg(src.meta + cells[q]) : zero4; };
-  auto cell_at = [&](uint32_t q) { return q < n_cells ? __ldg(cells + q) : kNoCell; };
-  auto meta_at = [&](uint32_t c) { return c != kNoCell ? __ldg(src.meta + c) : zero4; };
+  auto meta_of = [&](uint32_t q) { return q < n_cells ? src.meta[cells[q]] : zero4; };
+  auto cell_at = [&](uint32_t q) { return q < n_cells ? cells[q] : kNoCell; };
+  auto meta_at = [&](uint32_t c) { return c != kNoCell ? src.meta[c] : zero4; };
   uint4 md_next = meta_of(blk);
   uint4 md_after = meta_of(blk + G);
   uint32_t c_ahead = cell_at(blk + 2 * G);  // meta loaded one cell later
@@ -1248,15 +1248,15 @@ __device__ __forceinline__ void cellpass(const Pass& pass, const Grid* gp, const
       if (list_form) {
         // a cell whose stencil exceeds the staged form's limits: int32 lists,
         // neighbour records read from global memory
-        const int c = active ? min(__ldg(src.nn + a), src.max_nb) : 0;
+        const int c = active ? min(src.nn[a], src.max_nb) : 0;
         const uint32_t* row = src.nbr + a * src.max_nb;
         for (int k = sub; k < c; k += nsub)
-          pass.pair(T, pass.load(__ldg(row + k), tb.shift), g, acc);
+          pass.pair(T, pass.load(row[k], tb.shift), g, acc);
       } else {
         // the targets' staged-slot lists (ascending slots), kLC entries per
         // target at a time in shared memory, walked window by window
         if (tid < nr)
-          tot[tid] = min(r0 == 0 ? cur.nn : __ldg(src.nn + a0 + r0 + tid), src.max_nb);
+          tot[tid] = min(r0 == 0 ? cur.nn : src.nn[a0 + r0 + tid], src.max_nb);
         for (int lp = 0;; ++lp) {
           __syncthreads();  // tot written; the previous readers are done
           for (int i = tid; i < nr * (kLC / 4); i += kPT) {
@@ -1282,7 +1282,7 @@ __device__ __forceinline__ void cellpass(const Pass& pass, const Grid* gp, const
 #pragma unroll
               for (int i = 0; i < NJ; ++i) {
                 const int j = i * kPT + tid;
-                e[i] = pre ? cur.e[i] : (j < wn ? __ldg(es + j) : 0u);
+                e[i] = pre ? cur.e[i] : (j < wn ? es[j] : 0u);
               }
               // the entries' shift codes (5 bits each) kept packed across the wait
               static_assert(NJ <= 6, "shift codes packed into one register");
@@ -1436,10 +1436,10 @@ __device__ __forceinline__ void cellpipe(const Pass& pass, const Grid* gp, const
   const float4* shtab = tb.shift;
   const uint4 none = make_uint4(0u, kListForm, 0u, 0u);
   auto cell_at = [&](uint32_t qq) {
-    return qq < n0 ? __ldg(src.cells0 + qq)
-                   : (qq < n_cells ? __ldg(src.cells1 + (qq - n0)) : kNoCell);
+    return qq < n0 ? src.cells0[qq]
+                   : (qq < n_cells ? src.cells1[qq - n0] : kNoCell);
   };
-  auto meta_at = [&](uint32_t c) { return c != kNoCell ? __ldg(src.meta + c) : none; };
+  auto meta_at = [&](uint32_t c) { return c != kNoCell ? src.meta[c] : none; };
   auto present = [&](uint4 md) { return md.y != kListForm; };
   // staged entries of a cell's slots tid + u PT
   auto load_entries = [&](uint4 md, uint32_t* e) {
@@ -1447,7 +1447,7 @@ __device__ __forceinline__ void cellpipe(const Pass& pass, const Grid* gp, const
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int j = tid + u * PT;
-      e[u] = j < S ? __ldg(src.sent + md.x + (uint32_t)j) : 0u;
+      e[u] = j < S ? src.sent[md.x + (uint32_t)j] : 0u;
     }
   };
   auto issue_records = [&](uint4 md, const uint32_t* e, float4* rec) {
@@ -1472,11 +1472,11 @@ __device__ __forceinline__ void cellpipe(const Pass& pass, const Grid* gp, const
   auto count_of = [&](uint4 md) {
     if (kLists) {
       const int na = present(md) ? cell_na(md) : 0;
-      return tid < na ? min(__ldg(src.nn + md.z + tid), src.max_nb) : 0;
+      return tid < na ? min(src.nn[md.z + tid], src.max_nb) : 0;
     }
     int t, sub, nsub;
     target_of(md, t, sub, nsub);
-    return t >= 0 ? min(__ldg(src.nn + md.z + t), src.max_nb) : 0;
+    return t >= 0 ? min(src.nn[md.z + t], src.max_nb) : 0;
   };
   auto share_of = [&](uint4 md, int cnt) {
     Share sh;
@@ -1631,12 +1631,12 @@ __device__ __forceinline__ void cellpipe(const Pass& pass, const Grid* gp, const
         const int c = sh_cur.cnt;
         if (Pass::kPipePaired)
           for (; k + ns < c; k += 2 * ns)
-            pass.pair2(T_cur, pass.template fetch<W>(rec, __ldg(row + k)),
-                       pass.template fetch<W>(rec, __ldg(row + k + ns)), g, acc2);
+            pass.pair2(T_cur, pass.template fetch<W>(rec, row[k]),
+                       pass.template fetch<W>(rec, row[k + ns]), g, acc2);
         // the next entry's slot is loaded (through L1) while this pair is summed
-        int slot = k < c ? __ldg(row + k) : 0;
+        int slot = k < c ? row[k] : 0;
         for (; k < c; k += ns) {
-          const int nxt = k + ns < c ? __ldg(row + k + ns) : 0;
+          const int nxt = k + ns < c ? row[k + ns] : 0;
           pass.pair(T_cur, pass.template fetch<W>(rec, slot), g, acc);
           slot = nxt;
         }
