@@ -74,14 +74,16 @@ __device__ __forceinline__ void rel(const Grid& g, bool wrap, uint32_t e, float4
 // next group's load under way (a row streams from HBM once per pass and the
 // gathers wait for its entries: with the load at its use, momentum 184 us at
 // 250,047 particles and 4.23 ms in an ensemble of 5.7M, 166 us and 4.08 ms so).
+// Ordinary loads: the ensemble's one launch writes the rows anew in every step, and
+// the read-only path is for data that nobody writes during a launch.
 template <typename Body>
 __device__ __forceinline__ void for_entries(const uint32_t* row, int cnt, Body body) {
   const uint4* r4 = reinterpret_cast<const uint4*>(row);
   int k = 0;
-  uint4 nx = cnt > 0 ? __ldg(r4) : make_uint4(0, 0, 0, 0);
+  uint4 nx = cnt > 0 ? r4[0] : make_uint4(0, 0, 0, 0);
   for (; k + 4 <= cnt; k += 4) {
     const uint4 e = nx;
-    if (k + 4 < cnt) nx = __ldg(r4 + (k >> 2) + 1);
+    if (k + 4 < cnt) nx = r4[(k >> 2) + 1];
     body(e.x);
     body(e.y);
     body(e.z);
@@ -110,10 +112,10 @@ __device__ __forceinline__ void for_entries_part(const uint32_t* row, int cnt, i
     // the NSUB lanes of a target read NSUB consecutive entries at a time:
     // neighbours in the same cell, adjacent in memory, so a warp-wide gather
     // touches fewer lines (momentum 6.22 -> 6.11 ms at 8.4M particles)
-    uint32_t nx = sub < cnt ? __ldg(row + sub) : 0u;
+    uint32_t nx = sub < cnt ? row[sub] : 0u;
     for (int k = sub; k < cnt; k += NSUB) {
       const uint32_t e = nx;
-      if (k + NSUB < cnt) nx = __ldg(row + k + NSUB);
+      if (k + NSUB < cnt) nx = row[k + NSUB];
       body(e);
     }
     return;

@@ -1,8 +1,9 @@
 """Which loads take the read-only path (__ldg, const __restrict__ parameters).
 
 That path is for data nobody writes while the grid exists.  The kernels of a step's chain are
-scheduled while the one before them still runs (sph_launch.cuh), so a read-only load of what that
-one writes is a race that no run has to show; the sources are checked instead."""
+scheduled while the one before them still runs (sph_launch.cuh), and the ensemble's one launch
+writes its lists and records anew in every step, so a read-only load of what the kernel before, or
+the same launch, writes is a race that no run has to show; the sources are checked instead."""
 import os
 import re
 
@@ -19,6 +20,8 @@ ALLOWED = {
     "sph_pairs_fp64.cu": set(),
     "sph_lanes64.cuh": set(),
     "sph_sort.cu": {"org"},       # cell origins: written by k_zero_table, six kernels before
+    "sph_pairs32.cuh": set(),     # the ensemble's pair phases
+    "sph_ensemble.cu": {"A.hfac"},  # factor table: filled when the ensemble is made
     "sph_update.cu": {"hfac"},    # factor table: its kernel and k_update are ordered plainly
 }
 
