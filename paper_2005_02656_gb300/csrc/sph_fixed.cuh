@@ -182,11 +182,13 @@ SPH_FX void S6_d(double t, double& w, double& dw) {
 // one (v = 0 and subnormal v give 1 and are taken as zero by fixed()).
 SPH_FX int exp_above(double v) { return (int)((bits_of(v) >> 52) & 0x7ffu) + 1; }
 
-// v 2^(N - (eb - 1023)), |v| < 2^(eb - 1023); subnormals give zero.
+// v 2^(N - (eb - 1023)), |v| < 2^(eb - 1023); zero and subnormals give zero for
+// every eb (a zero vector has eb = 1, where shifting out the implicit bit would not do).
 template <int N>
 SPH_FX int64_t fixed(double v, int eb) {
   const uint64_t b = bits_of(v);
-  const int s = eb - (int)((b >> 52) & 0x7ffu);  // >= 1
+  const int f = (int)((b >> 52) & 0x7ffu);
+  const int s = f ? eb - f : 63;  // >= 1
   uint64_t m = (b & 0xfffffffffffffu) << (N - 52) | (uint64_t)1 << N;
   m >>= (unsigned)s < 63u ? s : 63;
   if (s <= 0) m = ((uint64_t)1 << N) - 1;  // |v| not below the power of two: the largest value
