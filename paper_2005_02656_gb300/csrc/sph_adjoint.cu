@@ -292,8 +292,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_momentum_a(Slot sl, Prep pr
     const int eca = sph::fix_matrix(sl.iad + 6 * a, cf);
     sph::fx::Vec3 Ca[3];
     sph::rows(cf, Ca);
-    // NaN where a matrix or g is not finite (their fixed-point forms are not)
-    const double nan_a = eca == 0 || eg > 2047 ? __longlong_as_double(0x7ff8000000000000LL) : 0.0;
     double xbx = 0, xby = 0, xbz = 0, vbx = 0, vby = 0, vbz = 0;
     double Xbar = 0, irbar = 0, cbar = 0;
     double Cbar[6] = {0, 0, 0, 0, 0, 0};
@@ -404,9 +402,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_momentum_a(Slot sl, Prep pr
                    sph::fx::scaled<true>(sph::fx::dot(Cb[1], Sb), kbs);
       double dbz = sph::fx::scaled<true>(sph::fx::dot(Ca[2], Sa), kas) +
                    sph::fx::scaled<true>(sph::fx::dot(Cb[2], Sb), kbs);
-      // a value that is not finite has no fixed-point form: NaN instead
-      if (max(max(ev, ecb == 0 ? 2048 : 0), max(esa, esb)) > 2047)
-        dbx = __longlong_as_double(0x7ff8000000000000LL);
       double r2b = (Pa * gca + Qa * vca) * dWa + (Pb * gcb + Qb * vcb) * dWb;
       double cpair = 0.0;
       if (on) {
@@ -443,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_adj_momentum_a(Slot sl, Prep pr
       rec[5] = make_double2(sby, sbz);
       pb.wk[slot] = make_double2(Wa, dWa);
     }
-    lanes_sum<NSUB>(xbx + nan_a, sums[0]);
+    lanes_sum<NSUB>(xbx, sums[0]);
     lanes_sum<NSUB>(xby, sums[1]);
     lanes_sum<NSUB>(xbz, sums[2]);
     lanes_sum<NSUB>(vbx, sums[3]);
@@ -668,13 +663,12 @@ __global__ void __launch_bounds__(kThreads) k_adj_iad(Slot sl, Prep pr, Work w, 
   const bool valid = p_pair < n;
   const int64_t p = valid ? p_pair : n - 1;
   const double xp = s.x[p], yp = s.y[p], zp = s.z[p];
-  const double nan = __longlong_as_double(0x7ff8000000000000LL);
   long long cf[6];
   sph::fx::Vec3 S[3];
   const int ep = sph::fix_matrix(w.Cb + 6 * p, cf);
   sph::rows(cf, S);
   const int ed = sph::fx::exp_above(2.0 * s.h[p]);  // |d| < 2 h_p
-  double xbx = ep == 0 ? nan : 0.0, xby = 0, xbz = 0;  // half of the adjoint of x_p
+  double xbx = 0, xby = 0, xbz = 0;  // half of the adjoint of x_p
   // p's own sum: pairs (p, b)
   const int cnt = valid ? min(sl.nn[p], mb) : 0;
   const uint32_t* list = sl.nbr + p * mb;
@@ -710,7 +704,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_iad(Slot sl, Prep pr, Work w, 
     ybx += wk.x * s0 + f * dx;
     yby += wk.x * s1 + f * dy;
     ybz += wk.x * s2 + f * dz;
-    volbar += ea == 0 ? nan : wbar * wk.x;
+    volbar += wbar * wk.x;
   }
   const double volp = pr.vol[p];
   lanes_sum<NSUB>(fma(volp, ybx, xbx), sums[0]);

@@ -179,8 +179,13 @@ SPH_FX void S6_d(double t, double& w, double& dw) {
 // with no carries: |X| < 2^61 leaves room for three terms.
 
 // Power of two above |v| for finite v, as the exponent field of a double plus
-// one (v = 0 and subnormal v give 1 and are taken as zero by fixed()).
+// one (v = 0 and subnormal v give 1 and are taken as zero by fixed()); 2048 for a
+// value that is not finite.
 SPH_FX int exp_above(double v) { return (int)((bits_of(v) >> 52) & 0x7ffu) + 1; }
+
+// In place of a power of two: a vector or matrix that is not finite.  fixed() makes
+// it zero, and scaled<true>() of a product that it enters gives NaN.
+constexpr int kNotFinite = 1 << 14;
 
 // v 2^(N - (eb - 1023)), |v| < 2^(eb - 1023); zero and subnormals give zero for
 // every eb (a zero vector has eb = 1, where shifting out the implicit bit would not do).
@@ -222,17 +227,20 @@ SPH_FX int64_t dot(const Vec3& a, const Vec3& b) {
 }
 
 // The double nearest to x 2^k; zero where that is below the normal range.  ANY:
-// infinity above it, for factors of any size (the forward pair sums, whose products
-// stay inside, would spend 2% on the compare).
+// infinity above it, and NaN past every finite vector's reach (kNotFinite), for factors
+// of any size (the forward pair sums, whose products stay inside, would spend 2% on the
+// compare).
 template <bool ANY = false>
 SPH_FX double scaled(int64_t x, int k) {
   const int64_t g = x >> 63;
   const uint64_t u = (uint64_t)((x ^ g) - g);
   const int z = clz64(u);
   const int f = 1085 + k - z;  // exponent field, less the implicit bit
-  if (u == 0 || (ANY ? (uint32_t)f > 2045u : f < 0))
+  if (u == 0 || (ANY ? (uint32_t)f > 2045u : f < 0)) {
+    if (ANY && f > kNotFinite / 2) return from_bits((uint64_t)0x7ff8000000000000);
     return ANY && u != 0 && f > 0
                ? from_bits((uint64_t)0x7ff0000000000000 | ((uint64_t)g << 63)) : 0.0;
+  }
   const uint64_t m = u << z;
   return from_bits((((uint64_t)(uint32_t)f << 52) + (m >> 11) + ((m >> 10) & 1u)) |
                    ((uint64_t)g << 63));

@@ -46,9 +46,10 @@ __device__ __forceinline__ void sep64(const Image64& im, double& dx, double& dy,
   }
 }
 
-// Power of two above three components (fx::exp_above; over 2047: not finite).
+// Power of two above three components (fx::exp_above), or fx::kNotFinite.
 __device__ __forceinline__ int exp_above3(double x, double y, double z) {
-  return max(fx::exp_above(x), max(fx::exp_above(y), fx::exp_above(z)));
+  const int e = max(fx::exp_above(x), max(fx::exp_above(y), fx::exp_above(z)));
+  return e <= 2047 ? e : fx::kNotFinite;
 }
 
 // A vector in block fixed point with the given power of two.
@@ -61,19 +62,20 @@ __device__ __forceinline__ fx::Vec3 vec64(double x, double y, double z, int eb) 
 }
 
 // C (6 entries) as block fixed point; the exponent field of the power of two
-// above its largest entry, or 0 where an entry is not finite.
+// above its largest entry, or fx::kNotFinite (and zero entries).
 __device__ __forceinline__ int fix_matrix(const double* C, long long cf[6]) {
   int eb = 1;
 #pragma unroll
   for (int q = 0; q < 6; ++q) eb = max(eb, fx::exp_above(C[q]));
+  if (eb > 2047) eb = fx::kNotFinite;
 #pragma unroll
   for (int q = 0; q < 6; ++q) cf[q] = fx::fixed<60>(C[q], eb);
-  return eb <= 2047 ? eb : 0;
+  return eb;
 }
 
 // 2^(eb - 1023) for eb of fix_matrix (not finite: NaN).
 __device__ __forceinline__ double power_of(int eb) {
-  if (eb == 0) return __longlong_as_double(0x7ff8000000000000LL);
+  if (eb == fx::kNotFinite) return __longlong_as_double(0x7ff8000000000000LL);
   return eb < 2047 ? __hiloint2double(eb << 20, 0) : 2.0 * __hiloint2double(2046 << 20, 0);
 }
 
