@@ -299,7 +299,8 @@ SPH_FX double times(const Mant& a, int64_t x, int k) {
 
 // v 2^kv / sqrt(R 2^kr) for v != 0 and R >= 2^52 (whose error of a unit is then
 // below 2^-52): y0 from the FP32 reciprocal square root, and the factor
-// 1 + e/2 + 3 e^2/8 with e = 1 - R y0^2, in 64-bit fixed point.
+// 1 + e/2 + 3 e^2/8 with e = 1 - R y0^2, in 64-bit fixed point.  Zero below 2^-900; the
+// callers' results end below 2^802.
 SPH_FX double over_root(int64_t v, int kv, uint64_t R, int kr) {
   int z = clz64(R);
   uint64_t m = R << z;  // m 2^-62 in [2, 4)

@@ -46,9 +46,14 @@ __device__ __forceinline__ void sep64(const Image64& im, double& dx, double& dy,
   }
 }
 
-// Power of two above three components (fx::exp_above), or fx::kNotFinite.
+// Power of two above three components (fx::exp_above; over 2047: not finite).
+__device__ __forceinline__ int exp_max3(double x, double y, double z) {
+  return max(fx::exp_above(x), max(fx::exp_above(y), fx::exp_above(z)));
+}
+
+// The same, or fx::kNotFinite.
 __device__ __forceinline__ int exp_above3(double x, double y, double z) {
-  const int e = max(fx::exp_above(x), max(fx::exp_above(y), fx::exp_above(z)));
+  const int e = exp_max3(x, y, z);
   return e <= 2047 ? e : fx::kNotFinite;
 }
 

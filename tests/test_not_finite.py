@@ -92,3 +92,74 @@ def test_a_seed_that_is_not_finite_reaches_every_adjoint_it_enters(row, value):
     for k in (3, 4, 5, 9):
         assert not np.isfinite(got[k][j]), k
     np.testing.assert_array_equal(got[:, far], want[:, far])
+
+
+def _sphere(speed):
+    """A sphere in homologous flow v = speed * x: every pair recedes (speed > 0) or approaches."""
+    s = sph_inputs.uniform_sphere(14, seed_index=80)
+    for k in "xyz":
+        s["v" + k] = speed * s[k]
+        s["v" + k + "h"] = s["v" + k].copy()
+    return s
+
+
+def _both(s, **opts):
+    from helpers import oracle_outputs
+    from paper_2005_02656_gb300 import SphSim
+    with np.errstate(all="ignore"):
+        _, _, ref = oracle_outputs(s, ng_target=0, max_nb=400)
+    sim = SphSim(s, ng_target=0, max_nb=400, **opts)
+    sim.find_neighbors()
+    sim.density()
+    sim.iad()
+    sim.momentum_energy()
+    got, flags = sim.to_numpy(), sim.error_word()
+    sim.close()
+    return got, ref, flags
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("speed", [1e200, 1e240, 1e280, 1e295])
+def test_receding_pairs_near_the_end_of_the_range(speed):
+    """Receding pairs have no viscosity: du = sum m W X v.C d stays in range and within the FP64
+    parity bound (1e-12 of the sum of magnitudes, which is linear in the speed without
+    viscosity), up to where v.C d itself ends."""
+    from helpers import oracle_outputs
+    got, ref, _ = _both(_sphere(speed))
+    _, _, unit = oracle_outputs(_sphere(1.0), ng_target=0, max_nb=400, alpha=0.0)
+    assert np.isfinite(ref["du"]).all() and np.isfinite(got["du"]).all()
+    assert (np.abs(got["du"] - ref["du"]) <= 1e-12 * speed * unit["sdu"]).all()
+    a = np.stack([got[k] - ref[k] for k in ("ax", "ay", "az")], 1)
+    assert (np.abs(a).max(1) <= 1e-12 * ref["sa"]).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("speed", [-1e200, -1e240, -1e280, -1e295])
+def test_approaching_pairs_past_the_range_overflow(speed):
+    """w^2 of Eq. 5 overflows: not finite and flagged, as in FP64."""
+    from paper_2005_02656_gb300 import _lib
+    got, ref, flags = _both(_sphere(speed))
+    assert flags & _lib.FLAG_NONFINITE
+    for k in ("ax", "ay", "az", "du"):
+        np.testing.assert_array_equal(np.isfinite(got[k]), np.isfinite(ref[k]))
+        assert not np.isfinite(got[k]).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf, 1e300])
+@pytest.mark.parametrize("opts", [{}, {"kernel_mode": "table"}])
+def test_one_velocity_that_is_not_finite(value, opts):
+    """Not finite where the plain sums are not, and the parity bound everywhere else."""
+    from paper_2005_02656_gb300 import _lib
+    s = sph_inputs.jittered_box(12, seed_index=81, vel_sigma=0.05)
+    s["vy"][17] = value
+    got, ref, flags = _both(s, **opts)
+    assert flags & _lib.FLAG_NONFINITE
+    for k in ("ax", "ay", "az", "du"):
+        fin = np.isfinite(ref[k])
+        np.testing.assert_array_equal(np.isfinite(got[k]), fin, err_msg=k)
+        assert fin.sum() > 0.5 * fin.size, k
+        scale = ref["sdu"] if k == "du" else ref["sa"]
+        if not opts:                     # (the oracle has the exact kernel here)
+            ok = fin & np.isfinite(scale)
+            assert (np.abs(got[k] - ref[k])[ok] <= 1e-12 * scale[ok]).all(), k
