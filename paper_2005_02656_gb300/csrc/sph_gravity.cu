@@ -27,6 +27,7 @@
 #include "sph_device.cuh"
 #include "sph_internal.cuh"
 #include "sph_scan.cuh"
+#include "sph_walk.cuh"
 
 namespace sph {
 namespace grav {
@@ -606,7 +607,6 @@ __global__ void __launch_bounds__(32 * kWalkWarps) k_walk(const Node* nodes, con
 // ms with 8 CTAs per SM (64 registers; 6 CTAs: 5.1 ms); whole call 7.95 -> 5.29 ms
 // (32 targets, scalar particles: 6.31 ms), 17,256 particles 1.15 -> 0.48 ms.
 constexpr int kTile32 = 16;
-constexpr int kStack32 = 384;
 
 struct Walk32Smem {
   int2 st[kStack32];   // nodes to visit
@@ -622,7 +622,8 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 8) k_walk32(const Node* nodes
                                                             const int64_t* n_nodes, StateView s,
                                                             int64_t n, Walk32Consts k32,
                                                             double* gx, double* gy, double* gz,
-                                                            unsigned long long* stats) {
+                                                            unsigned long long* stats,
+                                                            uint32_t* err) {
   __shared__ Walk32Smem smem[kWalkWarps];
   const int lane = threadIdx.x & 31, tl = lane % kTile32, half = lane / kTile32;
   Walk32Smem& W = smem[threadIdx.x >> 5];
@@ -675,10 +676,8 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 8) k_walk32(const Node* nodes
     if (lane == 0) W.st[0] = make_int2(root, (int)all);
     int sp = 1;
     __syncwarp();
-    while (sp > 0) {
-      // as many nodes as leave room for their children (at most 8 each) and for
-      // a depth-first walk from there (at most 7 more per level)
-      const int take = min(sp, min(32, max(1, (kStack32 - 64 - sp) / 7)));
+    while (walk_on(sp)) {
+      const int take = walk_take(sp);
       const bool have = lane < take;
       const int2 e = have ? W.st[sp - 1 - lane] : make_int2(0, 0);
       sp -= take;
@@ -814,6 +813,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 8) k_walk32(const Node* nodes
       }
       __syncwarp();
     }
+    if (sp > 0 && lane == 0) raise_flag(err, SPH_FLAG_CELL_OVERFLOW);
     nodes_used += used;
     pairs += npair;
     acc[0] -= px.x + px.y;
@@ -1001,7 +1001,7 @@ extern "C" int sph_gravity(sph_ctx* ctx, sph_state* state, double G, double eps,
     sph::grav::k_leaf_pairs<<<sph::grav::blocks_for(16 * n_occ, sm, 128), 128, 0, st>>>(
         nodes, n_occ, in, k32.sc, po);
     sph::grav::k_walk32<<<wb, 32 * sph::grav::kWalkWarps, 0, st>>>(
-        nodes, nf, po, n_nodes, in, n, k32, gx, gy, gz, stats);
+        nodes, nf, po, n_nodes, in, n, k32, gx, gy, gz, stats, ctx->err);
     ctx->launches += 3;
   } else {
     const int64_t tiles64 = (n + sph::grav::kTile64 - 1) / sph::grav::kTile64;
