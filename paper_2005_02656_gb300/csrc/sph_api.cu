@@ -494,7 +494,9 @@ int sph_density(sph_ctx* ctx, sph_state* state, sph_stream_t stream) {
   if (rc != SPH_OK) return rc;
   if (!ctx->have_lists)
     return sph::set_error(ctx, SPH_ERR_ORDER, "no neighbour lists: call sph_find_neighbors");
-  run_density(ctx, view_of(state), outs_of(state), state->n, (cudaStream_t)stream);
+  // (no particles, no launch: the device counters may be another search's)
+  if (state->n > 0)
+    run_density(ctx, view_of(state), outs_of(state), state->n, (cudaStream_t)stream);
   rc = finish(ctx, "sph_density");
   ctx->have_density = rc == SPH_OK;
   ctx->have_iad = 0;
@@ -505,7 +507,8 @@ int sph_iad(sph_ctx* ctx, sph_state* state, sph_stream_t stream) {
   int rc = check_state(ctx, state, true);
   if (rc != SPH_OK) return rc;
   if (!ctx->have_density) return sph::set_error(ctx, SPH_ERR_ORDER, "call sph_density first");
-  run_iad(ctx, view_of(state), outs_of(state), state->n, (cudaStream_t)stream);
+  if (state->n > 0)
+    run_iad(ctx, view_of(state), outs_of(state), state->n, (cudaStream_t)stream);
   rc = finish(ctx, "sph_iad");
   ctx->have_iad = rc == SPH_OK;
   return rc;
@@ -515,7 +518,8 @@ int sph_momentum_energy(sph_ctx* ctx, sph_state* state, sph_stream_t stream) {
   int rc = check_state(ctx, state, true);
   if (rc != SPH_OK) return rc;
   if (!ctx->have_iad) return sph::set_error(ctx, SPH_ERR_ORDER, "call sph_iad first");
-  run_momentum(ctx, view_of(state), outs_of(state), state->n, (cudaStream_t)stream);
+  if (state->n > 0)
+    run_momentum(ctx, view_of(state), outs_of(state), state->n, (cudaStream_t)stream);
   return finish(ctx, "sph_momentum_energy");
 }
 
