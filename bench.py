@@ -65,8 +65,8 @@ KERNEL_BYTES = {
              "iad": {"particle": 96, "slot": 0, "word": 0, "entry": 12},
              "momentum": {"particle": 168, "slot": 0, "word": 0, "entry": 12}},
 }
-# Per particle, the rest of the step (sort and gather 344, dt 16, update 244).
-OTHER_BYTES = 604
+# Per particle, the rest of the step (sort and gather 340, dt 16, update 244).
+OTHER_BYTES = 600
 PAIR_KERNELS = ("find", "density", "iad", "momentum")
 # The survey's step model: about 25 kflop and 1.9 KB of HBM traffic per
 # particle for the FP32-mixed step at 100 neighbours.

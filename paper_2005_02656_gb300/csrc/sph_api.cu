@@ -210,7 +210,7 @@ void free_all(sph_ctx* ctx) {
                   ctx->ktab32, ctx->code, ctx->slot,
                   ctx->perm_tmp, ctx->perm, ctx->tbl_count, ctx->tbl_start, ctx->occ,
                   ctx->scan_part, ctx->cell_of, ctx->s.x, ctx->s_id_buf, ctx->pos32,
-                  ctx->cell3, ctx->nn, ctx->nbr, ctx->wcache, ctx->vol, ctx->rec_d, ctx->rec_i,
+                  ctx->nn, ctx->nbr, ctx->wcache, ctx->vol, ctx->rec_d, ctx->rec_i,
                   ctx->rec_m, ctx->cmeta, ctx->sent, ctx->masks, ctx->salloc, ctx->cells, ctx->recA, ctx->recV,
                   ctx->recQ, ctx->recC, ctx->recC2, ctx->red.part, ctx->red.counter, ctx->stats,
                   ctx->hm_buf, ctx->hm_id, ctx->grav_buf};
@@ -361,7 +361,6 @@ int sph_init(const sph_params* params, int64_t n_max, sph_ctx** out) {
   ALLOC(sbuf, 13 * n);
   ALLOC(ctx->s_id_buf, n);
   ALLOC(ctx->pos32, n);
-  ALLOC(ctx->cell3, n);
   ALLOC(ctx->nn, n);
   ALLOC(ctx->nbr, (size_t)mb * n);
   if (params->precision == SPH_FP64) ALLOC(ctx->wcache, (size_t)mb * n);

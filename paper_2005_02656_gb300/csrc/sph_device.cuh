@@ -40,14 +40,6 @@ struct SincCoefs {
 constexpr int kSincTerms64 = 15;
 constexpr int kSincTerms32 = 7;
 
-__device__ __forceinline__ double sinc_poly64(double t) {
-  constexpr SincCoefs<kSincTerms64> C{};
-  double s = C.c[kSincTerms64 - 1];
-#pragma unroll
-  for (int k = kSincTerms64 - 2; k >= 0; --k) s = fma(s, t, C.c[k]);
-  return s;
-}
-
 // S(t) and dS/dt of the FP64 series (Horner on both).
 __device__ __forceinline__ void sinc_poly64_d(double t, double& S, double& dS) {
   constexpr SincCoefs<kSincTerms64> C{};
@@ -154,10 +146,6 @@ __device__ __forceinline__ double kernel_tdw_dt64(double t, double norm, int n) 
   return dW + t * d2W;
 }
 
-// W for t = v^2 < 4 (caller guarantees the neighbour criterion), norm = B_n/h^3.
-__device__ __forceinline__ double kernel_w64(double t, double norm, int n) {
-  return norm * ipow(sinc_poly64(t), n);
-}
 // t dW/dt (FP32), for the grad-h sum: v dW/dv = 2 t dW/dt.
 __device__ __forceinline__ float kernel_tdw32(float t, float norm, int n) {
   t = fminf(t, 4.0f);
@@ -193,9 +181,6 @@ __device__ __forceinline__ float2 kernel_w32x2(float2 t, float2 norm, int n) {
 }
 
 // The kernel of the context's mode: the series, or the table when tab != NULL.
-__device__ __forceinline__ double kw64(double t, double norm, int n, const double2* tab) {
-  return tab ? kernel_w64_tab(t, norm, tab) : kernel_w64(t, norm, n);
-}
 __device__ __forceinline__ float kw32(float t, float norm, int n, const float2* tab) {
   return tab ? kernel_w32_tab(t, norm, tab) : kernel_w32(t, norm, n);
 }
@@ -231,38 +216,6 @@ __device__ __forceinline__ bool exact_neighbor(const Grid& g, double xa, double 
 }
 
 __device__ __forceinline__ void raise_flag(uint32_t* err, uint32_t f) { atomicOr(err, f); }
-
-// Packed cell coordinates: 10 bits per axis.
-__device__ __forceinline__ int32_t pack_cell(int ix, int iy, int iz) {
-  return ix | (iy << 10) | (iz << 20);
-}
-__device__ __forceinline__ void unpack_cell(int32_t c, int& ix, int& iy, int& iz) {
-  ix = c & 1023;
-  iy = (c >> 10) & 1023;
-  iz = (c >> 20) & 1023;
-}
-
-// FP32 separation b - a along one axis from cell-relative offsets:
-// (off_b - off_a) + (cell_b - cell_a) * cs, with the cell difference taken
-// modulo the period and a final FP32 minimum image for grids of < 3 cells.
-__device__ __forceinline__ float sep32(float ob, float oa, int cb, int ca, const Grid& g, int ax) {
-  int dc = cb - ca;
-  if (g.periodic[ax]) {
-    int nc = g.nc[ax];
-    if (dc > nc / 2)
-      dc -= nc;
-    else if (dc < -(nc / 2))
-      dc += nc;
-  }
-  float d = fmaf((float)dc, g.cs32[ax], ob - oa);
-  if (g.periodic[ax]) {
-    if (d > g.halfL32[ax])
-      d -= g.L32[ax];
-    else if (d < -g.halfL32[ax])
-      d += g.L32[ax];
-  }
-  return d;
-}
 
 // Morton code of a cell: bit i of ix at 3i, iy at 3i+1, iz at 3i+2.
 __host__ __device__ __forceinline__ uint32_t spread3(uint32_t v) {
@@ -340,14 +293,6 @@ __device__ __forceinline__ double inv_root(double x) {
 }
 
 // --- reductions ---
-__device__ __forceinline__ double warp_min(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ double warp_max(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;

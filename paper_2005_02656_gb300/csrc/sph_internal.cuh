@@ -101,7 +101,6 @@ struct sph_ctx {
   // per-particle FP32 cell-relative data (sorted order)
   double* cell_org;     // cell origins lo + i cs per axis (3 x 2^kMaxCellBits)
   float4* pos32;        // offset from the cell origin (x, y, z) and h
-  int32_t* cell3;       // packed cell coordinates (10 bits per axis)
 
   // neighbour lists: nn[n], nbr[p * max_nb + k] = entry (sph_tile.cuh)
   int32_t* nn;
@@ -191,7 +190,7 @@ int cuda_fail(sph_ctx* ctx, cudaError_t e, const char* what);
 // Grid from the particles' extent + h_max; zero the cell table.
 void launch_grid(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st);
 // Counting sort by Morton cell code, deterministic order within cells; gathers
-// `in` into the sorted scratch ctx->s and builds pos32 / cell3 / cell_of.
+// `in` into the sorted scratch ctx->s and builds pos32 / cell_of.
 // Sort and gather: launch_sort (cells, order, first gather part) then
 // launch_gather_b (velocities, integrator history); launch_sort_gather does both.
 // wait_gather (may be null): an event the first gather part waits for (the
@@ -200,7 +199,7 @@ void launch_sort(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st,
                  cudaEvent_t wait_gather = nullptr);
 void launch_gather_b(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st);
 void launch_sort_gather(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st);
-// Recompute pos32 / cell3 for an already-sorted state (no permutation).
+// The 14 arrays of a state.
 void launch_copy_state(const StateView& dst, const StateView& src, int64_t n, cudaStream_t st,
                        sph_ctx* ctx);
 

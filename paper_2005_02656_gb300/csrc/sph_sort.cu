@@ -399,7 +399,7 @@ __device__ __forceinline__ uint32_t compact3(uint32_t v) {
 // memory round trip of its own.
 __global__ void k_gather_a(StateView in, StateView out, int64_t n, const double* org,
                            const int32_t* perm, const uint32_t* code, float4* pos32,
-                           int32_t* cell3, float4* rec_d) {
+                           float4* rec_d) {
   dep_enter();
   constexpr int kRow = 1 << kMaxCellBits;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -423,7 +423,6 @@ __global__ void k_gather_a(StateView in, StateView out, int64_t n, const double*
     out.u[p] = u;
     out.id[p] = id;
     pos32[p] = make_float4(ox, oy, oz, f32_rn(h));
-    cell3[p] = pack_cell(ix, iy, iz);
     rec_d[p] = make_float4(ox, oy, oz, f32_rn(m));
     s = s_next;
   }
@@ -519,7 +518,7 @@ void launch_sort(sph_ctx* ctx, const StateView& in, int64_t n, cudaStream_t st,
       ctx->tbl_count, ctx->perm_tmp, ctx->perm, ctx->cell_of);
   if (wait_gather) cudaStreamWaitEvent(st, wait_gather, 0);
   launch_dep(k_gather_a, pb, 256, 0, st, in, ctx->s, n, ctx->cell_org, ctx->perm, ctx->code,
-      ctx->pos32, ctx->cell3, ctx->rec_d);
+      ctx->pos32, ctx->rec_d);
   ctx->launches += 7;
 }
 
