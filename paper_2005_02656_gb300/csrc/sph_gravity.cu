@@ -424,7 +424,7 @@ __device__ __forceinline__ bool accept_mixed(const Node* nodes, const NodeF* nf,
 // The FP64 terms are evaluated from the rings, each lane taking its own next
 // term, so the FP64 pipe (which bounds the kernel, at 2 operations per clock
 // and SM; 86% busy) works on full warps: a warp that evaluates a term where it
-// meets it has 21 of its 32 lanes in it, because lanes that did not open the
+// meets it has 18 of its 32 lanes in it, because lanes that did not open the
 // parent or that open the node itself sit it out.  FP64 operations per node
 // term 42, per leaf particle 16 (G is applied once per target; inv_root).
 // Uniform sphere, theta = 0.5, whole call: 137,376 particles 28.6 -> 10.4 ms,

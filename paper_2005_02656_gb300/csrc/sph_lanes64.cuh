@@ -109,9 +109,12 @@ __device__ __forceinline__ void lanes_sum(double v, double* sums) {
 // Density + IAD + momentum with 4 / 8 / 16 lanes (us): 1,728 particles 167 / 103 /
 // 71, 4,096: 168 / 114 / 97, 8,000: 186 / 152 / 154, 13,824: 219 / 232 / 235,
 // 21,952: 357 / 338 / 337, 64,000: 800 / 803 / 884, 1.07M: 12,350 / 13,130 / -.
-// (At 32,768 four lanes take 451 against 457 us by themselves, but the step between
-// host copies 736 against 699.)  20 steps and their gradient (ms): 21.8 / 16.5 /
-// 16.6 at 4,096, 69.1 / 63.4 / 67.6 at 32,768, 180.5 / 181.6 / 203 at 110,592.
+// (At 13,824 four lanes are ahead: momentum's 432 blocks are one wave of up to 608,
+// with eight and sixteen lanes 1.4 and 2.8 waves, which no line in n follows; the first
+// line parts sixteen lanes from eight, level from 8,000 to 21,952 and 15% apart at 4,096.
+// At 32,768 four lanes take 451 against 457 us by themselves, but the step between host
+// copies 736 against 699.)  20 steps and their gradient (ms): 21.8 / 16.5 / 16.6 at 4,096,
+// 69.1 / 63.4 / 67.6 at 32,768, 180.5 / 181.6 / 203 at 110,592.
 inline int lanes64(int64_t n) { return n < 16384 ? 16 : n < 131072 ? 8 : 4; }
 
 // f(integral_constant<int, lanes>) for n particles.

@@ -6,7 +6,7 @@
 // added by a fixed butterfly.  Separations are FP64 minimum-image differences
 // of the positions.
 //
-// The FP64 pipe (2 operations per clock and SM) bounds these kernels (80-88% of
+// The FP64 pipe (2 operations per clock and SM) bounds these kernels (78-87% of
 // its cycles), so FP64 operations are what is saved:
 //  - S(v)^6 is evaluated on the integer pipes (sph_fixed.cuh) once per list
 //    entry by the density pass, kept without its factor B_n/h^3 (Lists64::w),
