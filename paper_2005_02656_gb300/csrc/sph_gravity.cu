@@ -423,7 +423,7 @@ __device__ __forceinline__ bool accept_mixed(const Node* nodes, const NodeF* nf,
 // its node terms and leaf particles each, added at the end by a fixed butterfly.
 // The FP64 terms are evaluated from the rings, each lane taking its own next
 // term, so the FP64 pipe (which bounds the kernel, at 2 operations per clock
-// and SM; 86% busy) works on full warps: a warp that evaluates a term where it
+// and SM; 87% busy) works on full warps: a warp that evaluates a term where it
 // meets it has 18 of its 32 lanes in it, because lanes that did not open the
 // parent or that open the node itself sit it out.  FP64 operations per node
 // term 42, per leaf particle 16 (G is applied once per target; inv_root).
@@ -603,9 +603,10 @@ __global__ void __launch_bounds__(32 * kWalkWarps) k_walk(const Node* nodes, con
 // broadcasts).  16 targets lie closer together than 32, so fewer nodes stay
 // undecided and fewer leaves are opened for some targets only: 1,660 leaf
 // particles per tile against 2,100, of which a target needs 730.
-// FP32 issue bounds the kernel.  998,317 particles, theta = 0.5: walk 7.10 -> 4.67
-// ms with 8 CTAs per SM (64 registers; 6 CTAs: 5.1 ms); whole call 7.95 -> 5.29 ms
-// (32 targets, scalar particles: 6.31 ms), 17,256 particles 1.15 -> 0.48 ms.
+// Instruction issue (71% of cycles) and the L1 data pipe (67%) bound the kernel.
+// 998,317 particles, theta = 0.5: walk 7.10 -> 4.67 ms with 8 CTAs per SM (64 registers;
+// 6 CTAs: 5.1 ms); whole call 7.95 -> 5.29 ms (32 targets, scalar particles: 6.31 ms),
+// 17,256 particles 1.15 -> 0.48 ms.
 constexpr int kTile32 = 16;
 
 struct Walk32Smem {

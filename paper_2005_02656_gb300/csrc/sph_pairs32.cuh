@@ -73,7 +73,7 @@ __device__ __forceinline__ void rel(const Grid& g, bool wrap, uint32_t e, float4
 // Calls body(entry) for the cnt entries of a row, reading 4 per 16-byte load, the
 // next group's load under way (a row streams from HBM once per pass and the
 // gathers wait for its entries: with the load at its use, momentum 184 us at
-// 250,047 particles and 4.23 ms in an ensemble of 5.7M, 166 us and 4.08 ms so).
+// 250,047 particles and 4.23 ms in an ensemble of 5.7M, 166 us and 4.16 ms so).
 // Ordinary loads: the ensemble's one launch writes the rows anew in every step, and
 // the read-only path is for data that nobody writes during a launch.
 template <typename Body>

@@ -19,7 +19,7 @@
 //    and 1/r, from the separation's fixed-point form;
 //  - the per-target work runs on whole warps (lanes_sum).
 // Per pair about 4 (density), 9 (IAD) and 26 (momentum) FP64 operations; at
-// 1.07M particles 1.82, 2.86 and 7.66 ms (7.99 with C_a applied to every pair),
+// 1.07M particles 1.82, 2.86 and 7.75 ms (7.99 with C_a applied to every pair),
 // where the FP64 series, products and comparisons with one thread per target took
 // 7.38, 4.11 and 20.6 ms.
 #include <cuda_runtime.h>

@@ -28,7 +28,9 @@ SPH_WALK int walk_take(int sp) {
 // walk_take takes fit.  A walk that ends with nodes left has overrun the stack, which
 // a tree of kLevels levels cannot; one comparison per turn guards it (a check at each
 // push took 2% of the call).
-SPH_WALK bool walk_on(int sp) { return (unsigned)(sp - 1) < (unsigned)(kStack32 - (kChildren - 1)); }
+SPH_WALK bool walk_on(int sp) {
+  return (unsigned)(sp - 1) < (unsigned)(kStack32 - (kChildren - 1));
+}
 
 }  // namespace grav
 }  // namespace sph
